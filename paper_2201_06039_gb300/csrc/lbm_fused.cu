@@ -352,8 +352,8 @@ k_fused_batch(DevParams P, const BatchInst* __restrict__ insts, const BatchItem*
 }
 
 // ================================================================ TMA producer / consumer kernel
-// Tile TX x TY.  Warps: producer, storer (FP32 only), compute warps (one tile node per thread:
-// pull, psi, collision), one halo warp (psi of the one-node ring around the tile).
+// Tile TX x TY.  Warps: copy warp (TMA loads and stores), compute warps (one tile node per thread:
+// pull, psi, collision), two halo warps (psi of the one-node ring around the tile).
 constexpr size_t align128(size_t v) { return (v + 127) / 128 * 128; }
 
 template <int TX_, int TY_, typename S_ = float> struct TmaShape {
@@ -361,15 +361,20 @@ template <int TX_, int TY_, typename S_ = float> struct TmaShape {
     static constexpr int kE = (int)sizeof(S);                        // bytes per stored population
     static constexpr int kInterior = TX_ * TY_;
     static constexpr int kHaloNodes = 2 * (TX_ + 2) + 2 * TY_;
-    static constexpr int kSlotsAll = kInterior + kHaloNodes;        // ring slots with a psi value
     static constexpr int kCompWarps = (kInterior + 31) / 32;         // one tile node per thread
-    static constexpr int kHaloWarps = 1;
-    static constexpr int kHaloPerLane = (kHaloNodes + 31) / 32;      // halo slots of one halo lane
+    // Two halo warps: with one, its three or four dependent pull-and-EOS passes a plane (32 of about
+    // 100 ring slots each) set the plane's time, as every plane ends at a barrier.  One copy warp in
+    // place of a producer and a storer makes room for the second at 128 registers a thread.  Pool of
+    // 200 x 200 x 300, 40 x 10 tiles: FP32 543 -> 516 us a step, BF16 597 -> 534; one 32 x 8 tile marching
+    // alone 2.2 -> 1.97 us a plane.
+    static constexpr int kHaloWarps = 2;
+    static constexpr int kHaloPerLane = (kHaloNodes + 63) / 64;      // halo slots of one halo lane
+    static_assert(kHaloPerLane == 2, "slots h and h + 64 of the ring");
     static constexpr int kCompThreads = kCompWarps * 32, kHaloThreads = kHaloWarps * 32;
     // Output path: the collided plane goes to an output tile in shared memory and leaves by TMA
-    // tensor stores issued by a storer warp (direct global stores by the compute threads measured
+    // tensor stores issued by the copy warp (direct global stores by the compute threads measured
     // slower, for FP32 and for 16-bit storage alike).
-    static constexpr int kLeadWarps = 2;                             // producer and storer warps first
+    static constexpr int kLeadWarps = 1;                             // the copy warp first
     static constexpr int kThreads = 32 * kLeadWarps + kCompThreads + kHaloThreads;
     // registers per thread: warp w runs on SM sub-partition w % 4, whose register file holds 16K
     // registers; the per-thread count goes in steps of 8
@@ -421,8 +426,7 @@ template <int TX_, int TY_, typename S_ = float> struct TmaShape {
     // thread counts of the named barriers (see k_fused_tma)
     static constexpr int kCntRing = kCompThreads + kHaloThreads + 32;
     static constexpr int kCntOut = kCompThreads + 32;
-    static constexpr int kCntEmpty = 64;
-    static_assert(kStages <= 4, "three named barriers a stage, ids 2..13");
+    static_assert(kStages <= 4, "two named barriers a stage, ids 2..9");
     static_assert(TX_ % 8 == 0 || kE == 4, "tile origins on 16-byte boundaries for 2-byte storage");
     static_assert(TX_ % 4 == 0, "tile origins on 16-byte boundaries");
     static_assert(kSmem <= 227 * 1024, "shared memory of one CTA");
@@ -582,11 +586,10 @@ __device__ __forceinline__ void stage_pulls(const DevParams& P, const typename S
 }
 
 // named barriers of the TMA kernel (bar.sync / bar.arrive; 0 is __syncthreads): the waiting
-// warps block in hardware and issue nothing while they wait.  Three per stage s (s < kStages <= 4).
+// warps block in hardware and issue nothing while they wait.  Two per stage s (s < kStages <= 4).
 constexpr int kBarComp = 1;
 __device__ __forceinline__ int bar_ring(int s) { return 2 + s; }
 __device__ __forceinline__ int bar_out_full(int s) { return 6 + s; }
-__device__ __forceinline__ int bar_empty(int s) { return 10 + s; }
 __device__ __forceinline__ void nb_sync(int id, int nthreads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
@@ -594,29 +597,29 @@ __device__ __forceinline__ void nb_arrive(int id, int nthreads) {
     asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 
-// Warp roles: warp 0 = producer (TMA loads), warp 1 = storer (TMA stores), then the compute warps
-// (thread t owns tile node t: it pulls the node's 26 populations once, writes the node's
-// (psi, rho) into the ring, keeps the populations in registers and collides the node one plane
-// later), then one halo warp (psi of the ring around the tile, kHaloPerLane slots a lane).
+// Warp roles: warp 0 = copies (TMA loads and stores), then the compute warps (thread t owns tile node
+// t: it pulls the node's 26 populations once, writes the node's (psi, rho) into the ring, keeps the
+// populations in registers and collides the node one plane later), then two halo warps (psi of the
+// ring around the tile, two slots a lane).
 // Stage use k (plane p) goes through stage s = k % kStages:
-//   full[s]        mbarrier: the TMA bytes of use k landed (producer -> compute, halo; bounded waits)
-//   RING(s)        named: producer bar.arrive once use k's loads are issued; compute and halo
+//   full[s]        mbarrier: the TMA bytes of use k landed (copy warp -> compute, halo; bounded waits)
+//   RING(s)        named: copy warp bar.arrive once use k's loads are issued; compute and halo
 //                  bar.sync once they have pulled plane p and put its psi into the ring.  After it
 //                  nobody reads the stage's window again, and the ring holds plane p.
-//   OUT_FULL(s)    named: compute bar.arrive -> storer bar.sync.  For the uses that carry an output
+//   OUT_FULL(s)    named: compute bar.arrive -> copy warp bar.sync.  For the uses that carry an output
 //                  (p = z0 + 1 .. z1 of an item) the compute warps first write the collided plane
-//                  p - 1 (and an edge tile's periodic images) into the stage itself.
-//   EMPTY(s)       named, bar.sync by storer and producer: the tensor stores have read the stage
-//                  and it may be refilled (the producer waits for use k before loading k + kStages).
+//                  p - 1 (and an edge tile's periodic images) into the stage itself; the copy warp
+//                  stores it, waits until the stores have read the stage and loads use k + kStages.
 // The collided plane thus leaves from the stage just pulled, so the compute warps never wait for
-// a store to drain: the storer and the next loads have kStages - 1 planes of time for it.
+// a store to drain: the copy warp has kStages - 1 planes of time for it.  One warp for both copies
+// needs no hand-off of the empty stage and leaves a warp's registers for the second halo warp.
 // Stage uses and ring planes follow one plane counter k across the CTA's items.  Every role runs
 // the same sequence of named-barrier operations whatever happens: an abort (a TMA wait that ran
 // out) skips only the mbarrier waits, the copies and the work, so no barrier is left incomplete.
-// No role laps another on a barrier: RING and EMPTY are synced by the roles that could run ahead
-// (compute, halo; storer, producer), the producer's next arrival on RING(s) follows its EMPTY(s)
-// sync of the previous use of s, and the compute warps' next arrival on OUT_FULL(s) follows their
-// RING(s) sync of the next use of s, which needs that arrival of the producer.
+// No role laps another on a barrier: RING is synced by the roles that could run ahead (compute,
+// halo); the copy warp's next arrival on RING(s) follows its OUT_FULL(s) sync of the previous use of
+// s, whose arrivals follow that use's RING(s); and the compute warps' next arrival on OUT_FULL(s)
+// follows their RING(s) sync of the next use of s, which needs that arrival of the copy warp.
 template <int TX_, int TY_, typename S, bool kWet>
 __global__ void __maxnreg__((TmaShape<TX_, TY_, S>::kMaxRegs))
 k_fused_tma(const __grid_constant__ CUtensorMap map14, const __grid_constant__ CUtensorMap map6,
@@ -662,94 +665,100 @@ k_fused_tma(const __grid_constant__ CUtensorMap map14, const __grid_constant__ C
     auto stage_of = [&](int s) { return reinterpret_cast<const S*>(smem_raw + (size_t)s * Sh::kStageOne); };
 
     if (warp == 0) {
-        // ------------------------------------------------------------ producer (lane 0 issues)
-        unsigned k = 0;
-        for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
+        // ------------------------------------------------------------ copies (lane 0 issues)
+        // a position in the CTA's sequence of stage uses: plane p of an item
+        struct Use {
+            int item, x0, y0, z0, z1, p;
+        };
+        auto enter = [&](Use& u, int item) {
             const int chunk = item / ntiles, tile = item % ntiles;
-            const int x0 = (tile % tiles_x) * TX_, y0 = (tile / tiles_x) * TY_;
-            const int z0 = chunk * zchunk, z1 = min(P.nz, z0 + zchunk);
-            // window origin in storage coordinates: (x0 - kXOff) + kGX, (y0 - 2) + kGY
-            const int cx = x0 - Sh::kXOff + kGX, cy = y0;
-            for (int p = z0 - 1; p <= z1; ++p, ++k) {
-                const int s = k % kStages;
-                if (k >= (unsigned)kStages) nb_sync(bar_empty(s), Sh::kCntEmpty);   // use k - kStages stored
-                if (lane == 0) {
-                    if (P.test_stall && k == 0) {
-                        // timeout-path test: the first stage's data never comes; the producer waits
-                        // (bounded) on a barrier nothing completes, then releases the stage empty
-                        if (!mbar_wait(&stall_bar, 0u)) {
-                            abort_flag = 1;
-                            atomicOr(flag, 2);
-                        }
-                        mbar_arrive(&full_bar[s]);
-                    } else if (abort_flag) {
-                        mbar_arrive(&full_bar[s]);   // release the waiters without data
-                    } else {
-                        const int mz = map_coord(p, P.nz, P.bc[4], P.bc[5]);
-                        const int zu = src_plane_up(P, mz), zd = src_plane_dn(P, mz);
-                        const unsigned bytes =
-                            (14u + (zu >= 0 ? 6u : 0u) + (zd >= 0 ? 6u : 0u)) * (unsigned)(Sh::kWin * Sh::kE);
-                        unsigned char* st = smem_raw + (size_t)s * Sh::kStageOne;
-                        mbar_expect_tx(&full_bar[s], bytes);
-                        tma_load_4d(st, &map14, cx, cy, mz, 0, &full_bar[s]);
-                        if (zu >= 0) tma_load_4d(st + Sh::kGrp1, &map6, cx, cy, zu, 14, &full_bar[s]);
-                        if (zd >= 0) tma_load_4d(st + Sh::kGrp2, &map6, cx, cy, zd, 20, &full_bar[s]);
+            u.item = item;
+            u.x0 = (tile % tiles_x) * TX_;
+            u.y0 = (tile / tiles_x) * TY_;
+            u.z0 = chunk * zchunk;
+            u.z1 = min(P.nz, u.z0 + zchunk);
+            u.p = u.z0 - 1;
+        };
+        auto next = [&](Use& u) {
+            if (++u.p > u.z1) enter(u, u.item + gridDim.x);
+        };
+        Use ld, st;
+        enter(ld, blockIdx.x);
+        enter(st, blockIdx.x);
+        unsigned kl = 0, k = 0;   // stage uses loaded, stored
+        auto load = [&]() {
+            const int s = kl % kStages;
+            if (lane == 0) {
+                if (P.test_stall && kl == 0) {
+                    // timeout-path test: the first stage's data never comes; the copy warp waits
+                    // (bounded) on a barrier nothing completes, then releases the stage empty
+                    if (!mbar_wait(&stall_bar, 0u)) {
+                        abort_flag = 1;
+                        atomicOr(flag, 2);
                     }
+                    mbar_arrive(&full_bar[s]);
+                } else if (abort_flag) {
+                    mbar_arrive(&full_bar[s]);   // release the waiters without data
+                } else {
+                    // window origin in storage coordinates: (x0 - kXOff) + kGX, (y0 - 2) + kGY
+                    const int cx = ld.x0 - Sh::kXOff + kGX, cy = ld.y0;
+                    const int mz = map_coord(ld.p, P.nz, P.bc[4], P.bc[5]);
+                    const int zu = src_plane_up(P, mz), zd = src_plane_dn(P, mz);
+                    const unsigned bytes =
+                        (14u + (zu >= 0 ? 6u : 0u) + (zd >= 0 ? 6u : 0u)) * (unsigned)(Sh::kWin * Sh::kE);
+                    unsigned char* sb = smem_raw + (size_t)s * Sh::kStageOne;
+                    mbar_expect_tx(&full_bar[s], bytes);
+                    tma_load_4d(sb, &map14, cx, cy, mz, 0, &full_bar[s]);
+                    if (zu >= 0) tma_load_4d(sb + Sh::kGrp1, &map6, cx, cy, zu, 14, &full_bar[s]);
+                    if (zd >= 0) tma_load_4d(sb + Sh::kGrp2, &map6, cx, cy, zd, 20, &full_bar[s]);
                 }
-                __syncwarp();
-                nb_arrive(bar_ring(s), Sh::kCntRing);   // use k is under way
             }
-        }
-        // the last stage uses (every use of EMPTY is matched on both sides)
-        const unsigned q0 = k > (unsigned)kStages ? k - kStages : 0u;
-        for (unsigned q = q0; q < k; ++q) nb_sync(bar_empty(q % kStages), Sh::kCntEmpty);
-        // copies still in flight land before the CTA exits (every use completes one phase; bounded)
-        if (lane == 0)
-            for (unsigned q = q0; q < k; ++q) mbar_wait(&full_bar[q % kStages], (q / kStages) & 1);
-        __syncwarp();
-    } else if (warp == 1) {
-        // ------------------------------------------------------------ storer (lane 0 issues)
-        unsigned k = 0;
-        for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
-            const int chunk = item / ntiles, tile = item % ntiles;
-            const int x0 = (tile % tiles_x) * TX_, y0 = (tile / tiles_x) * TY_;
-            const int z0 = chunk * zchunk, z1 = min(P.nz, z0 + zchunk);
-            // box (x, slot, y, z) at the tile origin (x a multiple of 4 floats); the last tile
-            // row uses the map whose box holds exactly its rows, so a box never reaches past
-            // ny; columns beyond nx fall outside the tensor and are not written
-            const CUtensorMap* m = y0 + TY_ > P.ny ? &map_out_top : &map_out;
-            // ghost cells written from this tile (storage coordinates; every box lies inside
-            // the padded plane exactly): its 4 edge columns to the opposite ghost columns, its
-            // 2 edge rows to the opposite ghost rows, and the corner block
-            const bool left = ghosts == 1 && x0 == 0, right = ghosts == 1 && x0 + TX_ >= P.nx;
-            const bool bottom = ghosts == 1 && y0 == 0, top = ghosts == 1 && y0 + TY_ >= P.ny;
-            const int gx_col = right ? kGX - kGW : P.nx + kGX;    // destination of the column box
-            const int gy_row = top ? kGY - 2 : P.ny + kGY;        // destination of the row box
-            const CUtensorMap* mc = y0 + TY_ > P.ny ? &map_gcol_top : &map_gcol;
-            const CUtensorMap* mr = x0 + TX_ > P.nx ? &map_grow_right : &map_grow;
+            __syncwarp();
+            nb_arrive(bar_ring(s), Sh::kCntRing);   // use kl is under way
+            next(ld);
+            ++kl;
+        };
+        for (int s = 0; s < kStages && ld.item < n_items; ++s) load();
+        for (; st.item < n_items; next(st), ++k) {
+            const int s = k % kStages;
+            nb_sync(bar_out_full(s), Sh::kCntOut);
             // ghost mode 2, nx no multiple of the 16-byte band: the last tile column stores its
             // nodes itself (a tensor store clipped at nx inside a 16-byte unit also writes the
             // ghost columns past nx, which the first tile column's nodes write)
-            const bool direct_tile = ghosts == 2 && x0 + TX_ > P.nx && P.nx % kGW != 0;
-            for (int p = z0 - 1; p <= z1; ++p, ++k) {
-                const int s = k % kStages;
-                nb_sync(bar_out_full(s), Sh::kCntOut);
-                if (p > z0 && lane == 0 && !abort_flag && !direct_tile) {   // the stage holds collided plane p - 1
-                    const int z = p - 1;
-                    unsigned char* st = smem_raw + (size_t)s * Sh::kStageOne;
-                    tma_store_4d(m, st, x0 + kGX, 0, y0 + kGY, z);
-                    if (left || right) tma_store_4d(mc, st + Sh::kGColOff, gx_col, 0, y0 + kGY, z);
-                    if (top || bottom) tma_store_4d(mr, st + Sh::kGRowOff, x0 + kGX, 0, gy_row, z);
+            const bool direct_tile = ghosts == 2 && st.x0 + TX_ > P.nx && P.nx % kGW != 0;
+            if (st.p > st.z0 && lane == 0 && !abort_flag && !direct_tile) {   // the stage holds collided plane p - 1
+                const int z = st.p - 1, x0 = st.x0, y0 = st.y0;
+                // box (x, slot, y, z) at the tile origin (x a multiple of 4 floats); the last tile
+                // row uses the map whose box holds exactly its rows, so a box never reaches past
+                // ny; columns beyond nx fall outside the tensor and are not written
+                unsigned char* sb = smem_raw + (size_t)s * Sh::kStageOne;
+                tma_store_4d(y0 + TY_ > P.ny ? &map_out_top : &map_out, sb, x0 + kGX, 0, y0 + kGY, z);
+                if (ghosts == 1) {
+                    // ghost cells written from this tile (storage coordinates; every box lies inside
+                    // the padded plane exactly): its 4 edge columns to the opposite ghost columns, its
+                    // 2 edge rows to the opposite ghost rows, and the corner block
+                    const bool left = x0 == 0, right = x0 + TX_ >= P.nx, bottom = y0 == 0, top = y0 + TY_ >= P.ny;
+                    const int gx_col = right ? kGX - kGW : P.nx + kGX;    // destination of the column box
+                    const int gy_row = top ? kGY - 2 : P.ny + kGY;        // destination of the row box
+                    if (left || right)
+                        tma_store_4d(y0 + TY_ > P.ny ? &map_gcol_top : &map_gcol, sb + Sh::kGColOff, gx_col, 0, y0 + kGY, z);
+                    if (top || bottom)
+                        tma_store_4d(x0 + TX_ > P.nx ? &map_grow_right : &map_grow, sb + Sh::kGRowOff, x0 + kGX, 0, gy_row, z);
                     if ((left || right) && (top || bottom))
-                        tma_store_4d(&map_gcor, st + Sh::kGCorOff, gx_col, 0, gy_row, z);
-                    bulk_commit();
-                    bulk_wait_read_all();
+                        tma_store_4d(&map_gcor, sb + Sh::kGCorOff, gx_col, 0, gy_row, z);
                 }
-                __syncwarp();
-                nb_sync(bar_empty(s), Sh::kCntEmpty);   // the stage may be refilled
+                bulk_commit();
+                bulk_wait_read_all();
             }
+            __syncwarp();
+            if (ld.item < n_items) load();   // the stage may be refilled
         }
-        if (lane == 0) bulk_wait_all();   // the stores have completed before the CTA exits
+        if (lane == 0) {
+            bulk_wait_all();   // the stores have completed before the CTA exits
+            // ... and copies still in flight after an abort (every use completes one phase; bounded)
+            for (unsigned q = k > (unsigned)kStages ? k - kStages : 0u; q < k; ++q)
+                mbar_wait(&full_bar[q % kStages], (q / kStages) & 1);
+        }
         __syncwarp();
     } else if (warp < Sh::kLeadWarps + Sh::kCompWarps) {
         // ------------------------------------------------------------ compute
@@ -927,42 +936,49 @@ k_fused_tma(const __grid_constant__ CUtensorMap map14, const __grid_constant__ C
         if (bad) atomicOr(flag, 1);
         finish_sums<kComp>(partial, n_items, counter, sums_next, ct, kBarComp, red_a, red_b, &is_last);
     } else {
-        // ------------------------------------------------------------ halo psi (one warp)
+        // ------------------------------------------------------------ halo psi (two warps)
+        const int h = tid - 32 * (Sh::kLeadWarps + Sh::kCompWarps);
         int bad = 0;
         unsigned k = 0;
+        int lx[2], ly[2];   // ring slots h and h + 64
+#pragma unroll
+        for (int j = 0; j < 2; ++j) tma_slot_of<TX_, TY_>(Sh::kInterior + h + 64 * j, lx[j], ly[j]);
         for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
             const int chunk = item / ntiles, tile = item % ntiles;
             const int x0 = (tile % tiles_x) * TX_, y0 = (tile / tiles_x) * TY_;
             const int z0 = chunk * zchunk, z1 = min(P.nz, z0 + zchunk);
+            // per slot: lattice coordinates (-1: none), ring offset and window cell, once an item
+            int mx[2], my[2], roff[2], woff[2];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int gx = x0 + lx[j] - 1, gy = y0 + ly[j] - 1;
+                const bool used = lx[j] >= 0 && gx <= P.nx && gy <= P.ny;
+                mx[j] = used ? map_coord(gx, P.nx, P.bc[0], P.bc[1]) : -1;
+                my[j] = used ? map_coord(gy, P.ny, P.bc[2], P.bc[3]) : 0;
+                roff[j] = used ? bbase(P, ly[j] * Sh::kRingW + lx[j], 0, 0, kRP) : 0;
+                woff[j] = used ? bbase(P, (ly[j] + 1) * kWinW + lx[j] - 1 + Sh::kXOff, -(kWinW + 1), kWinW + 1, Sh::kWin) : 0;
+            }
             for (int p = z0 - 1; p <= z1; ++p, ++k) {
                 const int s = k % kStages;
                 float2* rp = ring + (k % kRing) * kRP;
                 wait_full(s, (k / kStages) & 1);
                 const S* st = stage_of(s);
                 const int mz = map_coord(p, P.nz, P.bc[4], P.bc[5]);
-                // kHaloPerLane slots a lane, rolled (one copy of the pull and EOS code); the slot
-                // geometry is recomputed per plane rather than kept in an indexed array
+                // both slots in turn, rolled (one copy of the pull and EOS code)
 #pragma unroll 1
-                for (int j = 0; j < Sh::kHaloPerLane; ++j) {
-                    const int q = Sh::kInterior + lane + 32 * j;
-                    if (q >= Sh::kSlotsAll) break;
-                    int lx, ly;
-                    tma_slot_of<TX_, TY_>(q, lx, ly);
-                    const int gx = x0 + lx - 1, gy = y0 + ly - 1;
-                    if (gx < -1 || gx > P.nx || gy < -1 || gy > P.ny) continue;
-                    const int mx = map_coord(gx, P.nx, P.bc[0], P.bc[1]);
-                    const int my = map_coord(gy, P.ny, P.bc[2], P.bc[3]);
-                    const int roff = bbase(P, ly * Sh::kRingW + lx, 0, 0, kRP);
+                for (int j = 0; j < 2; ++j) {
+                    const int x = j ? mx[1] : mx[0], y = j ? my[1] : my[0];
+                    if (x < 0) continue;
+                    float2* const out = rp + (j ? roff[1] : roff[0]);
                     if (kWet && p < 0) {   // virtual (psi, rho) of the solid layer below a wetting -z wall
-                        rp[roff] = wall_entry(P, mx, my);
+                        *out = wall_entry(P, x, y);
                         continue;
                     }
                     float f[19], g[7];
-                    stage_pulls<Sh>(P, st + bbase(P, (ly + 1) * kWinW + lx - 1 + Sh::kXOff, -(kWinW + 1), kWinW + 1, Sh::kWin),
-                                    src, mx, my, mz, f, g);
+                    stage_pulls<Sh>(P, st + (j ? woff[1] : woff[0]), src, x, y, mz, f, g);
                     const float rho = sum19(f), T = sum7(g);
                     const float psi2 = psi_squared(P, rho, T);
-                    rp[roff] = make_float2(psi_of(psi2), rho);
+                    *out = make_float2(psi_of(psi2), rho);
                     bad |= !(psi2 > 0.f) || !isfinite(rho) || !isfinite(T);
                 }
                 nb_sync(bar_ring(s), Sh::kCntRing);   // the window is read; the ring holds plane p
