@@ -434,9 +434,8 @@ bool gb300lbm::build_tma_maps(const DevParams& d, int precision, void* buf0, voi
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return false;
     if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) return false;
     int shape = -1, zchunk = 0, items = 0;
-    tma_plan_for(d, model_ctas > 0 ? model_ctas : sms, forced_shape, forced_zchunk, &shape, &zchunk, &items);
+    tma_plan_for(d, model_ctas > 0 ? model_ctas : sms, forced_shape, forced_zchunk, max_items, &shape, &zchunk, &items);
     if (shape < 0 || (size_t)optin < tma_smem_bytes(shape, precision)) return false;
-    if (items > max_items) return false;
     void* fn = nullptr;
     cudaDriverEntryPointQueryResult q;
     if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||

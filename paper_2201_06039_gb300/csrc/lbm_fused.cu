@@ -1044,22 +1044,31 @@ __global__ void __launch_bounds__(256) k_ghosts(DevParams P, S* __restrict__ pop
 }
 
 // Tile shapes of the TMA kernel (index = plan shape): 8 to 13 compute warps of one tile node a
-// thread.  kTmaRate is each shape's node rate per CTA relative to 32 x 8 (a prior for the model
-// below, which lbm_autotune replaces by measurement).  The 40-wide shapes tile lattices whose nx
-// is a multiple of 40 (such as 200) without a partial tile column.
+// thread.  kTmaRate is each shape's node rate per CTA relative to 32 x 8, measured (a plane of a tile
+// takes 1.75, 2.3, 2.26, 2.51, 2.4, 2.53 us on the pool, 1.97 us for one 32 x 8 tile alone).  The 40-wide
+// shapes tile lattices whose nx is a multiple of 40 (such as 200) without a partial tile column.
 #define GB300_TMA_SHAPES(M) M(0, 32, 8) M(1, 40, 7) M(2, 32, 12) M(3, 24, 16) M(4, 40, 8) M(5, 40, 10)
 constexpr int kNumTmaShapes = 6;
 constexpr int kTmaTX[kNumTmaShapes] = {32, 40, 32, 24, 40, 40};
 constexpr int kTmaTY[kNumTmaShapes] = {8, 7, 12, 16, 8, 10};
-constexpr double kTmaRate[kNumTmaShapes] = {1.0, 1.0, 1.25, 1.12, 1.1, 1.25};
+constexpr double kTmaRate[kNumTmaShapes] = {1.0, 0.97, 1.17, 1.06, 1.08, 1.11};
 
-// Plan of the TMA kernel for a lattice: the tile shape and z-chunking with the least modelled
-// time of the busiest CTA.  Items (tile, z-chunk) go round robin to the persistent CTAs; a plane
-// of an item costs its tile nodes over the shape's rate, and an item about two planes more (its
-// two psi-only planes and the pipeline's fill).  forced_shape / forced_zchunk (>= 0 / > 0) pin
-// either choice.  lbm_autotune replaces the model by measurement.
-void tma_plan(const DevParams& P, int ctas, int forced_shape, int forced_zchunk, int* shape, int* zchunk,
-              int* items) {
+// Modelled time of a plan: items (tile, z-chunk) go round robin to the persistent CTAs; a plane of an
+// item costs its tile nodes over the shape's rate, and an item two planes more (its psi-only planes).
+// The busiest CTA counts.  The model holds down to chunks of one plane: a 32^3 lattice measured
+// 45.6, 28.0, 19.3, 15.1, 13.8 us a step at chunks of 16, 8, 4, 2, 1 planes (8 to 128 items on 152
+// SMs), 64 x 64 x 96 42.8, 36.0, 40.5, 50.0 us at 16, 12, 6, 3 planes (96, 128, 256, 512 items), so
+// small lattices take the shortest chunks that still make one round of items.
+// (The tenth of a plane stands for an item's change-over: of equal splits the one of longer items.)
+double tma_cost(int shape, long long items, int zc, int ctas) {
+    return (double)((items + ctas - 1) / ctas) * kTmaTX[shape] * kTmaTY[shape] / kTmaRate[shape] * (zc + 2.1);
+}
+
+// Plan of the TMA kernel for a lattice: the tile shape and z-chunking of least modelled time among
+// those of at most max_items items.  forced_shape / forced_zchunk (>= 0 / > 0) pin either choice.
+// lbm_autotune replaces the model by measurement.
+void tma_plan(const DevParams& P, int ctas, int forced_shape, int forced_zchunk, int max_items, int* shape,
+              int* zchunk, int* items) {
     double best = -1.0;
     *shape = -1;
     for (int sh = 0; sh < kNumTmaShapes; ++sh) {
@@ -1069,12 +1078,9 @@ void tma_plan(const DevParams& P, int ctas, int forced_shape, int forced_zchunk,
         for (int nch = 1; nch <= P.nz; ++nch) {
             int zc = (P.nz + nch - 1) / nch;
             if (forced_zchunk > 0) zc = forced_zchunk < P.nz ? forced_zchunk : P.nz;
-            const int nchunks = (P.nz + zc - 1) / zc;
-            if (forced_zchunk <= 0 && zc < 16 && nch > 1) break;
-            const long long n = (long long)tiles * nchunks;
-            const long long per_cta = (n + ctas - 1) / ctas;
-            const double cost = (double)per_cta * tx * ty / kTmaRate[sh] * (zc + 2.0);
-            if (best < 0 || cost < best) {
+            const long long n = (long long)tiles * ((P.nz + zc - 1) / zc);
+            const double cost = tma_cost(sh, n, zc, ctas);
+            if (n <= max_items && (best < 0 || cost < best)) {
                 best = cost;
                 *shape = sh;
                 *zchunk = zc;
@@ -1137,17 +1143,16 @@ size_t tma_smem_bytes(int shape, int precision) {
     return (size_t)-1;
 }
 
-void tma_plan_for(const DevParams& P, int ctas, int forced_shape, int forced_zchunk, int* shape, int* zchunk,
-                  int* items) {
-    tma_plan(P, ctas, forced_shape, forced_zchunk, shape, zchunk, items);
+void tma_plan_for(const DevParams& P, int ctas, int forced_shape, int forced_zchunk, int max_items, int* shape,
+                  int* zchunk, int* items) {
+    tma_plan(P, ctas, forced_shape, forced_zchunk, max_items, shape, zchunk, items);
 }
 
 int tma_num_shapes() { return kNumTmaShapes; }
 double tma_rate(int shape) { return kTmaRate[shape]; }
 
 int tma_zchunk_candidates(const DevParams& P, int ctas, int shape, int* zcs, int max) {
-    // the z-chunks of the shape in increasing modelled cost (distinct, at least 16 planes unless
-    // the column is shorter), the whole column included
+    // the z-chunks of the shape in increasing modelled cost (distinct), the whole column included
     const int tx = kTmaTX[shape], ty = kTmaTY[shape];
     const long long tiles = (long long)((P.nx + tx - 1) / tx) * ((P.ny + ty - 1) / ty);
     int n = 0;
@@ -1155,10 +1160,8 @@ int tma_zchunk_candidates(const DevParams& P, int ctas, int shape, int* zcs, int
     int zc_of[64];
     for (int nch = 1; nch <= P.nz && n < 64; ++nch) {
         const int zc = (P.nz + nch - 1) / nch;
-        if (zc < 16 && nch > 1) break;
         if (n > 0 && zc_of[n - 1] == zc) continue;
-        const long long items = tiles * ((P.nz + zc - 1) / zc);
-        cost[n] = (double)((items + ctas - 1) / ctas) * (zc + 2.0);
+        cost[n] = tma_cost(shape, tiles * ((P.nz + zc - 1) / zc), zc, ctas);
         zc_of[n++] = zc;
     }
     int out = 0;

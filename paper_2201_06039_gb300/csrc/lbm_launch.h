@@ -84,9 +84,10 @@ bool tma_eligible(const DevParams& P, int precision);
 cudaError_t launch_ghosts(const DevParams& P, int precision, void* pops, cudaStream_t s);
 // tile shapes 0: 32 x 8, 1: 40 x 7, 2: 32 x 12, 3: 24 x 16 (window boxes tma_box_w x tma_box_h per
 // population slot)
-// forced_shape >= 0 / forced_zchunk > 0 pin the shape / the z-chunk of the plan
-void tma_plan_for(const DevParams& P, int ctas, int forced_shape, int forced_zchunk, int* shape, int* zchunk,
-                  int* items);
+// forced_shape >= 0 / forced_zchunk > 0 pin the shape / the z-chunk of the plan; plans of more than
+// max_items items are not considered (*shape -1 if none is left)
+void tma_plan_for(const DevParams& P, int ctas, int forced_shape, int forced_zchunk, int max_items, int* shape,
+                  int* zchunk, int* items);
 int tma_num_shapes();
 // the plan model's node rate of a tile shape (relative to 32 x 8)
 double tma_rate(int shape);
