@@ -219,79 +219,72 @@ __device__ __forceinline__ float wall_T(const DevParams& P, int face, int x, int
     return T;
 }
 
-template <typename S, int A>
-__device__ __forceinline__ float pull_f_one(const DevParams& P, const S* __restrict__ src, int i,
-                                            int x, int y, int z, const Nbr& n) {
+// Storage offset from a node to the pull source x - e_a, and whether the pull crosses a face of the
+// axis masks (fbb: bounce back, gabb: anti-bounce back).
+template <int A> __device__ __forceinline__ int pull_off(const DevParams& P, int x, int y, int z, const Nbr& n) {
     constexpr int ex = ex19(A), ey = ey19(A), ez = ez19(A);
-    if (A != 0 && crosses<A>(n.fbb))   // Eq. 50: f_a(x_b, t+1) = f*_{abar}(x_b, t)
-        return Codec<S>::load(src + (size_t)fslot(opp(A)) * P.Ns + bidx(P, i, P.Nidx), P.shift_f[opp(A)]);
-    int s = sidx(P, src_c(ex, x, n.xm, n.xp), src_c(ey, y, n.ym, n.yp), src_c(ez, z, n.zm, n.zp));
-    return Codec<S>::load(src + (size_t)fslot(A) * P.Ns + bidx(P, s, P.Nidx), P.shift_f[A]);
+    return (src_c(ex, x, n.xm, n.xp) - x) + P.Rs * (src_c(ey, y, n.ym, n.yp) - y) +
+           P.splane * (src_c(ez, z, n.zm, n.zp) - z);
+}
+template <typename S>
+__device__ __forceinline__ float load_at(const DevParams& P, const S* __restrict__ src, int slot, int i, float shift) {
+    return Codec<S>::load(src + (size_t)slot * P.Ns + bidx(P, i, P.Nidx), shift);
 }
 
-// Node at least one node away from every face: every pull source is i - (ex + nx ey + nx ny ez).
-__device__ __forceinline__ bool deep_interior(const DevParams& P, int x, int y, int z) {
-    return (unsigned)(x - 1) < (unsigned)(P.nx - 2) && (unsigned)(y - 1) < (unsigned)(P.ny - 2) &&
-           (unsigned)(z - 1) < (unsigned)(P.nz - 2);
+// Pull of f_a.  kWalls: a lane whose link crosses a wall reads f*_abar of its own node (Eq. 50:
+// f_a(x_b, t+1) = f*_abar(x_b, t)) by selecting slot and offset, so that the warp issues one load;
+// w_abar = w_a, so the storage shift is the same.
+template <typename S, int A, bool kWalls>
+__device__ __forceinline__ float pull_f_one(const DevParams& P, const S* __restrict__ src, int i, int x, int y, int z,
+                                            const Nbr& n) {
+    const int off = pull_off<A>(P, x, y, z, n);
+    const bool back = kWalls && A != 0 && crosses<A>(n.fbb);
+    return load_at<S>(P, src, back ? fslot(opp(A)) : fslot(A), back ? i : i + off, P.shift_f[A]);
 }
 
-template <typename S, int A>
-__device__ __forceinline__ float pull_f_fast(const DevParams& P, const S* __restrict__ src, int i) {
-    constexpr int ex = ex19(A), ey = ey19(A), ez = ez19(A);
-    return Codec<S>::load(src + (size_t)fslot(A) * P.Ns + bidx(P, i - ex - ey * P.Rs - ez * P.splane, P.Nidx),
-                          P.shift_f[A]);
-}
-
-// Pull of all 19 f (pull != 0) or direct read of the node's own values (fresh state).
+// Pull of all 19 f (pull != 0) or direct read of the node's own values (fresh state).  One code path
+// for every lane of a warp: the offsets take care of periodic and clamped faces, and warps without a
+// wall link skip the selection.  (With a separate path for nodes away from every face, each warp that
+// held a face node ran both: at nx = 64 that is every warp.)
 template <typename S>
 __device__ __forceinline__ void load_f(const DevParams& P, const S* __restrict__ src, int pull, int i,
                                        int x, int y, int z, const Nbr& n, float f[19]) {
-    if (pull && deep_interior(P, x, y, z)) {
-#define GB300_PULL(A) f[A] = pull_f_fast<S, A>(P, src, i);
-        GB300_PULL(0) GB300_PULL(1) GB300_PULL(2) GB300_PULL(3) GB300_PULL(4) GB300_PULL(5)
-        GB300_PULL(6) GB300_PULL(7) GB300_PULL(8) GB300_PULL(9) GB300_PULL(10) GB300_PULL(11)
-        GB300_PULL(12) GB300_PULL(13) GB300_PULL(14) GB300_PULL(15) GB300_PULL(16) GB300_PULL(17)
-        GB300_PULL(18)
-#undef GB300_PULL
-    } else if (pull) {
-#define GB300_PULL(A) f[A] = pull_f_one<S, A>(P, src, i, x, y, z, n);
-        GB300_PULL(0) GB300_PULL(1) GB300_PULL(2) GB300_PULL(3) GB300_PULL(4) GB300_PULL(5)
-        GB300_PULL(6) GB300_PULL(7) GB300_PULL(8) GB300_PULL(9) GB300_PULL(10) GB300_PULL(11)
-        GB300_PULL(12) GB300_PULL(13) GB300_PULL(14) GB300_PULL(15) GB300_PULL(16) GB300_PULL(17)
-        GB300_PULL(18)
+#define GB300_PULLS(W)                                                                                              \
+    GB300_PULL(0, W) GB300_PULL(1, W) GB300_PULL(2, W) GB300_PULL(3, W) GB300_PULL(4, W) GB300_PULL(5, W)           \
+    GB300_PULL(6, W) GB300_PULL(7, W) GB300_PULL(8, W) GB300_PULL(9, W) GB300_PULL(10, W) GB300_PULL(11, W)         \
+    GB300_PULL(12, W) GB300_PULL(13, W) GB300_PULL(14, W) GB300_PULL(15, W) GB300_PULL(16, W) GB300_PULL(17, W)     \
+    GB300_PULL(18, W)
+    if (pull) {
+#define GB300_PULL(A, W) f[A] = pull_f_one<S, A, W>(P, src, i, x, y, z, n);
+        if (__any_sync(__activemask(), n.fbb != 0u)) {
+            GB300_PULLS(true)
+        } else {
+            GB300_PULLS(false)
+        }
 #undef GB300_PULL
     } else {
 #pragma unroll
-        for (int a = 0; a < 19; ++a) f[a] = Codec<S>::load(src + (size_t)fslot(a) * P.Ns + bidx(P, i, P.Nidx), P.shift_f[a]);
+        for (int a = 0; a < 19; ++a) f[a] = load_at<S>(P, src, fslot(a), i, P.shift_f[a]);
     }
 }
 
+// Pull of g_a on the D3Q7 velocities; a link that crosses a face not periodic for g takes Eq. 51:
+// g_a(x_b, t+1) = -g+_abar(x_b, t) + 2 w_abar T_w (w_abar = w_a on D3Q7).
 template <typename S, int A>
-__device__ __forceinline__ float pull_g_one(const DevParams& P, const S* __restrict__ src, int i,
-                                            int x, int y, int z, const Nbr& n) {
+__device__ __forceinline__ float pull_g_one(const DevParams& P, const S* __restrict__ src, int i, int x, int y, int z,
+                                            const Nbr& n) {
     constexpr int ex = ex7(A), ey = ey7(A), ez = ez7(A);
     constexpr int face = ex > 0 ? 0 : ex < 0 ? 1 : ey > 0 ? 2 : ey < 0 ? 3 : ez > 0 ? 4 : 5;
-    if (A != 0 && (n.gabb & (1u << face))) {
-        // Eq. 51: g_a(x_b, t+1) = -g+_{abar}(x_b, t) + 2 w_abar T_w   (w_abar = w_a on D3Q7)
-        float gp = Codec<S>::load(src + (size_t)gslot(opp(A)) * P.Ns + bidx(P, i, P.Nidx), P.shift_g[opp(A)]);
-        return -gp + 2.f * P.w1 * wall_T(P, face, x, y);
-    }
-    int s = sidx(P, src_c(ex, x, n.xm, n.xp), src_c(ey, y, n.ym, n.yp), src_c(ez, z, n.zm, n.zp));
-    return Codec<S>::load(src + (size_t)gslot(A) * P.Ns + bidx(P, s, P.Nidx), P.shift_g[A]);
+    const int off = pull_off<A>(P, x, y, z, n);   // the D3Q7 velocities are the first seven of D3Q19
+    const bool back = A != 0 && (n.gabb & (1u << face)) != 0u;
+    const float v = load_at<S>(P, src, back ? gslot(opp(A)) : gslot(A), back ? i : i + off, P.shift_g[A]);
+    return back ? -v + 2.f * P.w1 * wall_T(P, face, x, y) : v;
 }
 
 template <typename S>
 __device__ __forceinline__ void load_g(const DevParams& P, const S* __restrict__ src, int pull, int i,
                                        int x, int y, int z, const Nbr& n, float g[7]) {
-    if (pull && deep_interior(P, x, y, z)) {
-        g[0] = Codec<S>::load(src + (size_t)gslot(0) * P.Ns + bidx(P, i, P.Nidx), P.shift_g[0]);
-        g[1] = Codec<S>::load(src + (size_t)gslot(1) * P.Ns + bidx(P, i - 1, P.Nidx), P.shift_g[1]);
-        g[2] = Codec<S>::load(src + (size_t)gslot(2) * P.Ns + bidx(P, i + 1, P.Nidx), P.shift_g[2]);
-        g[3] = Codec<S>::load(src + (size_t)gslot(3) * P.Ns + bidx(P, i - P.Rs, P.Nidx), P.shift_g[3]);
-        g[4] = Codec<S>::load(src + (size_t)gslot(4) * P.Ns + bidx(P, i + P.Rs, P.Nidx), P.shift_g[4]);
-        g[5] = Codec<S>::load(src + (size_t)gslot(5) * P.Ns + bidx(P, i - P.splane, P.Nidx), P.shift_g[5]);
-        g[6] = Codec<S>::load(src + (size_t)gslot(6) * P.Ns + bidx(P, i + P.splane, P.Nidx), P.shift_g[6]);
-    } else if (pull) {
+    if (pull) {
         g[0] = pull_g_one<S, 0>(P, src, i, x, y, z, n);
         g[1] = pull_g_one<S, 1>(P, src, i, x, y, z, n);
         g[2] = pull_g_one<S, 2>(P, src, i, x, y, z, n);
@@ -301,7 +294,7 @@ __device__ __forceinline__ void load_g(const DevParams& P, const S* __restrict__
         g[6] = pull_g_one<S, 6>(P, src, i, x, y, z, n);
     } else {
 #pragma unroll
-        for (int a = 0; a < 7; ++a) g[a] = Codec<S>::load(src + (size_t)gslot(a) * P.Ns + bidx(P, i, P.Nidx), P.shift_g[a]);
+        for (int a = 0; a < 7; ++a) g[a] = load_at<S>(P, src, gslot(a), i, P.shift_g[a]);
     }
 }
 
@@ -617,7 +610,7 @@ __host__ __device__ constexpr float w19(int a) { return a == 0 ? 1.f / 3.f : a <
 // Pull of g_a on the D3Q19 velocities: g_a(x, t+1) = g+_a(x - e_a, t), or, where x - e_a lies
 // behind a face that is not periodic for g, Eq. 51 at the node itself:
 // g_a(x, t+1) = -g+_abar(x, t) + 2 w_a T_w (the face of the highest axis crossed gives T_w).
-template <typename S, int A>
+template <typename S, int A, bool kFaces>
 __device__ __forceinline__ float pull_g19_one(const DevParams& P, const S* __restrict__ src, int i, int x, int y,
                                               int z, const Nbr& n) {
     constexpr int ex = ex19(A), ey = ey19(A), ez = ez19(A);
@@ -625,28 +618,28 @@ __device__ __forceinline__ float pull_g19_one(const DevParams& P, const S* __res
     const bool cx = ex > 0 ? (n.gabb & 1u) : ex < 0 ? (n.gabb & 2u) : 0u;
     const bool cy = ey > 0 ? (n.gabb & 4u) : ey < 0 ? (n.gabb & 8u) : 0u;
     const bool cz = ez > 0 ? (n.gabb & 16u) : ez < 0 ? (n.gabb & 32u) : 0u;
-    if (A != 0 && (cx || cy || cz)) {
-        const int face = cz ? (ez > 0 ? 4 : 5) : cy ? (ey > 0 ? 2 : 3) : (ex > 0 ? 0 : 1);
-        const float gp = Codec<S>::load(src + (size_t)gslot19(opp(A)) * P.Ns + bidx(P, i, P.Nidx), 0.f);
-        return -gp + 2.f * w19(A) * wall_T(P, face, x, y);
-    }
-    const int s = sidx(P, src_c(ex, x, n.xm, n.xp), src_c(ey, y, n.ym, n.yp), src_c(ez, z, n.zm, n.zp));
-    return Codec<S>::load(src + (size_t)gslot19(A) * P.Ns + bidx(P, s, P.Nidx), 0.f);
+    const bool back = kFaces && A != 0 && (cx || cy || cz);
+    const int off = pull_off<A>(P, x, y, z, n);
+    const float v = load_at<S>(P, src, back ? gslot19(opp(A)) : gslot19(A), back ? i : i + off, 0.f);
+    if (!back) return v;
+    const int face = cz ? (ez > 0 ? 4 : 5) : cy ? (ey > 0 ? 2 : 3) : (ex > 0 ? 0 : 1);
+    return -v + 2.f * w19(A) * wall_T(P, face, x, y);
 }
 
 template <typename S>
 __device__ __forceinline__ void load_g19(const DevParams& P, const S* __restrict__ src, int pull, int i, int x,
                                          int y, int z, const Nbr& n, float g[19]) {
     if (pull) {
-#define GB300_PULL(A) g[A] = pull_g19_one<S, A>(P, src, i, x, y, z, n);
-        GB300_PULL(0) GB300_PULL(1) GB300_PULL(2) GB300_PULL(3) GB300_PULL(4) GB300_PULL(5)
-        GB300_PULL(6) GB300_PULL(7) GB300_PULL(8) GB300_PULL(9) GB300_PULL(10) GB300_PULL(11)
-        GB300_PULL(12) GB300_PULL(13) GB300_PULL(14) GB300_PULL(15) GB300_PULL(16) GB300_PULL(17)
-        GB300_PULL(18)
+#define GB300_PULL(A, W) g[A] = pull_g19_one<S, A, W>(P, src, i, x, y, z, n);
+        if (__any_sync(__activemask(), n.gabb != 0u)) {
+            GB300_PULLS(true)
+        } else {
+            GB300_PULLS(false)
+        }
 #undef GB300_PULL
     } else {
 #pragma unroll
-        for (int a = 0; a < 19; ++a) g[a] = Codec<S>::load(src + (size_t)gslot19(a) * P.Ns + bidx(P, i, P.Nidx), 0.f);
+        for (int a = 0; a < 19; ++a) g[a] = load_at<S>(P, src, gslot19(a), i, 0.f);
     }
 }
 

@@ -39,7 +39,10 @@ template <int TY, int QT = 7> struct FusedShape {
     static constexpr int kRingW = TX + 2, kRingH = TY + 2;
     static constexpr int kRingPlane = kRingW * kRingH;
     static constexpr size_t kStageFloats = (size_t)kPops * kInterior;
-    static constexpr size_t kSmemBytes = 2 * kStageFloats * sizeof(float) + 3 * kRingPlane * sizeof(float2);
+    // ring of four (psi, rho) planes: z - 1, z, z + 1 of the collision and the plane being filled, so
+    // that one barrier a plane is enough
+    static constexpr int kRing = 4;
+    static constexpr size_t kSmemBytes = 2 * kStageFloats * sizeof(float) + kRing * kRingPlane * sizeof(float2);
 };
 
 // coordinate of the node whose (psi, rho) fills a ring slot at coordinate c (may be -1 or n):
@@ -184,7 +187,7 @@ __device__ __forceinline__ void fused_column(const DevParams& P, const S* __rest
     auto psi_pass = [&](int zp) {
         if (!slot_used) return;
         if (kWet && zp < 0 && P.wet) {   // solid layer below a wetting -z wall: virtual (psi, rho)
-            ring[((zp + 3) % 3) * Sh::kRingPlane + slot] = wall_entry(P, mx, my);
+            ring[((zp + 4) % Sh::kRing) * Sh::kRingPlane + slot] = wall_entry(P, mx, my);
             return;
         }
         const bool in_chunk = zp >= z0 && zp < z1;
@@ -196,7 +199,7 @@ __device__ __forceinline__ void fused_column(const DevParams& P, const S* __rest
         Therm<QT>::template load<S>(P, src, pull_g, i, mx, my, mz, n, g);
         float rho = sum19(f), T = Therm<QT>::sum(g);
         float psi2 = psi_squared(P, rho, T);
-        ring[((zp + 3) % 3) * Sh::kRingPlane + slot] = make_float2(psi_of(psi2), rho);
+        ring[((zp + 4) % Sh::kRing) * Sh::kRingPlane + slot] = make_float2(psi_of(psi2), rho);
         if (owner && in_chunk) {
             float* st = stage + ((zp - z0) & 1) * Sh::kStageFloats + tid;
 #pragma unroll
@@ -220,9 +223,9 @@ __device__ __forceinline__ void fused_column(const DevParams& P, const S* __rest
 #pragma unroll
         for (int a = 0; a < QT; ++a) g[a] = st[(19 + a) * Sh::kInterior];
         float rho = sum19(f), T = Therm<QT>::sum(g);
-        const float2* rm = ring + ((z + 2) % 3) * Sh::kRingPlane;
-        const float2* r0 = ring + (z % 3) * Sh::kRingPlane;
-        const float2* rp = ring + ((z + 1) % 3) * Sh::kRingPlane;
+        const float2* rm = ring + ((z + 3) % Sh::kRing) * Sh::kRingPlane;
+        const float2* r0 = ring + (z % Sh::kRing) * Sh::kRingPlane;
+        const float2* rp = ring + ((z + 1) % Sh::kRing) * Sh::kRingPlane;
         const float2 me = r0[slot];
         RingStencil rs = ring_stencil(rm, r0, rp, bbase(P, slot, -(Sh::kRingW + 1), Sh::kRingW + 1, Sh::kRingPlane),
                                       Sh::kRingW);
@@ -242,12 +245,10 @@ __device__ __forceinline__ void fused_column(const DevParams& P, const S* __rest
 
     psi_pass(z0 - 1);
     psi_pass(z0);
-    __syncthreads();
     for (int z = z0; z < z1; ++z) {
         psi_pass(z + 1);
         __syncthreads();
         collide(z);
-        __syncthreads();
     }
 }
 
@@ -259,7 +260,7 @@ k_fused(DevParams P, const S* __restrict__ src, S* __restrict__ dst, int pull_f,
     using Sh = FusedShape<TY, QT>;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     float* stage = reinterpret_cast<float*>(smem_raw);                       // [2][26][TY][32]
-    float2* ring = reinterpret_cast<float2*>(stage + 2 * Sh::kStageFloats);  // [3][TY+2][34]
+    float2* ring = reinterpret_cast<float2*>(stage + 2 * Sh::kStageFloats);  // [4][TY+2][34]
     __shared__ double red_a[Sh::kThreads / 32], red_b[Sh::kThreads / 32];
     __shared__ int is_last;
 
