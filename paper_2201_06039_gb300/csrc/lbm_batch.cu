@@ -6,13 +6,13 @@
 //             slots layout of a single lattice, so the per-instance set-up and read-out kernels
 //             run unchanged on the instance's block)
 //   phis      phi_s history, instances concatenated (node offset field_off_k)
-//   psirho    (psi, rho) scratch of the largest instance (read-out only)
+//   psirho    (psi, rho) scratch of the largest instance (totals only)
 //   sums      (sum rho, sum T) per instance: two ping-pong sets (rho_ave of the next step) and
 //             one set for lbm_batch_get_totals
 //   partial   one double2 per work item (and per block of the read-out reductions)
 //   counters  work counter + ticket of the batched kernel, ticket of the read-out reductions
 //   flag      non-finite / timeout flag
-//   insts     BatchInst table, items: BatchItem table of the current plan
+//   insts     BatchInst table, items: BatchItem table of the current plan, ritems: of the read-out
 //
 // Plan: tile rows (4 or 8 of the 32-wide tile) and the number of z-chunks per column.  Items of
 // one instance are contiguous; instances are ordered by size, largest first, so that the atomic
@@ -71,8 +71,9 @@ struct lbm_batch {
     int max_N, max_items, max_partial;
     cudaStream_t stream, capture, launch;
     char* base;
-    size_t off_pops[2], off_phis, off_psirho, off_sums, off_partial, off_counters, off_flag, off_inst, off_items;
+    size_t off_pops[2], off_phis, off_psirho, off_sums, off_partial, off_counters, off_flag, off_inst, off_items, off_ritems;
     int plan, n_items, ctas, sms;
+    int n_ritems;                      // items of the read-out table
     int cur, slot;
     bool fresh_f, fresh_g, first, initialised;
     long long steps;
@@ -95,6 +96,7 @@ struct lbm_batch {
     float* phis() { return (float*)(base + off_phis); }
     BatchInst* d_inst() { return (BatchInst*)(base + off_inst); }
     BatchItem* d_items() { return (BatchItem*)(base + off_items); }
+    BatchItem* d_ritems() { return (BatchItem*)(base + off_ritems); }
     // StateBufs of instance k (read-out kernels) or of the whole batch (k < 0)
     StateBufs bufs(int k) {
         const size_t pb = pop_bytes(p.precision);
@@ -148,6 +150,18 @@ int items_of_plan(const lbm_batch* b, const Plan& pl, std::vector<BatchItem>* it
                 }
     }
     return count;
+}
+
+// Items of the one-launch read-out: 32 x 8 tiles and chunks of 16 planes (two of the 18 planes a block
+// reads are read by the next block too), instances largest first.
+void readout_items(const lbm_batch* b, std::vector<BatchItem>* items) {
+    for (int idx = 0; idx < b->n; ++idx) {
+        const int k = b->order[idx];
+        const DevParams& d = b->dps[k];
+        for (int z = 0; z < d.nz; z += 16)
+            for (int y = 0; y < d.ny; y += 8)
+                for (int x = 0; x < d.nx; x += 32) items->push_back(BatchItem{k, x, y, z, std::min(d.nz, z + 16), 0});
+    }
 }
 
 void drop_batch_graphs(lbm_batch* b) {
@@ -478,6 +492,10 @@ int lbm_batch_create(const lbm_params* common, int n_instances, const int* dims,
     b->off_flag = take(sizeof(int));
     b->off_inst = take(sizeof(BatchInst) * (size_t)n_instances);
     b->off_items = take(sizeof(BatchItem) * (size_t)b->max_items);
+    std::vector<BatchItem> ritems;
+    readout_items(b, &ritems);
+    b->n_ritems = (int)ritems.size();
+    b->off_ritems = take(sizeof(BatchItem) * ritems.size());
     b->stream = (cudaStream_t)common->cuda_stream;
     b->launch = b->stream;
     b->capture = nullptr;
@@ -500,6 +518,7 @@ int lbm_batch_create(const lbm_params* common, int n_instances, const int* dims,
     for (auto& d : b->dps) d.check_flag = (int*)(b->base + b->off_flag);
     e = cudaMemsetAsync(b->base + b->off_sums, 0, b->off_inst - b->off_sums, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+    if (e == cudaSuccess) e = cudaMemcpy(b->d_ritems(), ritems.data(), sizeof(BatchItem) * ritems.size(), cudaMemcpyHostToDevice);
     int rc = e == cudaSuccess ? set_plan(b, 0) : fail(LBM_ECUDA, "initial memset: %s", cudaGetErrorString(e));
     if (rc) {
         cudaFree(b->base);
@@ -677,15 +696,10 @@ int lbm_batch_get_moments(lbm_batch* b, float* rho, float* ux, float* uy, float*
     bool dev[5];
     for (int q = 0; q < 5; ++q) dev[q] = outs[q] && is_device_ptr(outs[q]);
     float* stage = (float*)b->pbuf(b->cur ^ 1);   // overwritten by the next step anyway
-    for (int k = 0; k < b->n; ++k) {
-        StateBufs B = b->bufs(k);
-        const size_t fo = (size_t)b->inst[k].field_off;
-        float* dst[5];
-        for (int q = 0; q < 5; ++q) dst[q] = outs[q] ? (dev[q] ? outs[q] : stage + q * N) + fo : nullptr;
-        GB300_CK(launch_psi(b->dps[k], b->p.precision, B, nullptr, b->stream));
-        GB300_CK(launch_moments(b->dps[k], b->p.precision, B, b->sums(b->slot) + 2 * k, dst[0], dst[1], dst[2],
-                                dst[3], dst[4], b->stream));
-    }
+    float* dst[5];
+    for (int q = 0; q < 5; ++q) dst[q] = outs[q] ? (dev[q] ? outs[q] : stage + q * N) : nullptr;
+    GB300_CK(launch_readout_batch(b->dps[0], b->p.precision, b->d_inst(), b->d_ritems(), b->n_ritems, b->bufs(-1),
+                                  b->sums(b->slot), dst[0], dst[1], dst[2], dst[3], dst[4], b->stream));
     for (int q = 0; q < 5; ++q)
         if (outs[q] && !dev[q])
             GB300_CK(cudaMemcpyAsync(outs[q], stage + q * N, N * 4, cudaMemcpyDeviceToHost, b->stream));

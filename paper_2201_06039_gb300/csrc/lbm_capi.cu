@@ -693,13 +693,12 @@ int lbm_get_moments(lbm_ctx* c, float* rho, float* ux, float* uy, float* uz, flo
     // u carries F_m / 2: a scheme-1 wetting wall's virtual densities must be those of this state
     if (c->dp.wet && c->dp.wet_scheme == 1)
         CK(launch_wall_table(c->dp, c->p.precision, B.src, B.pull_f, (float2*)(c->base + c->L.wall), c->stream));
-    CK(launch_psi(c->dp, c->p.precision, B, nullptr, c->stream));
     // outputs staged in the population buffer the next step overwrites anyway
     float* stage = (float*)c->pbuf(c->cur ^ 1);
     float* outs[5] = {rho, ux, uy, uz, T};
     float* dst[5];
     for (int k = 0; k < 5; ++k) dst[k] = outs[k] ? (is_device_ptr(outs[k]) ? outs[k] : stage + k * N) : nullptr;
-    CK(launch_moments(c->dp, c->p.precision, B, c->sums(c->slot), dst[0], dst[1], dst[2], dst[3], dst[4], c->stream));
+    CK(launch_readout(c->dp, c->p.precision, B, c->sums(c->slot), dst[0], dst[1], dst[2], dst[3], dst[4], c->stream));
     for (int k = 0; k < 5; ++k)
         if (outs[k] && dst[k] != outs[k])
             CK(cudaMemcpyAsync(outs[k], dst[k], N * 4, cudaMemcpyDeviceToHost, c->stream));

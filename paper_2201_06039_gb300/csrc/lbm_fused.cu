@@ -21,6 +21,9 @@
 //               TMA tensor stores, 16-bit planes through direct stores of the collision threads.
 //               Persistent CTAs take (z-chunk, tile) items round robin.
 #include <cuda.h>
+
+#include <algorithm>
+
 #include "lbm_launch.h"
 
 namespace gb300lbm {
@@ -281,6 +284,23 @@ k_fused(DevParams P, const S* __restrict__ src, S* __restrict__ dst, int pull_f,
 }
 
 // ================================================================ batched ensemble
+// Parameters of one instance of an ensemble: the shared model constants with its geometry.
+__device__ __forceinline__ DevParams instance_params(const DevParams& P, const BatchInst& I) {
+    DevParams Q = P;
+    Q.nx = I.nx; Q.ny = I.ny; Q.nz = I.nz;
+    Q.plane = I.nx * I.ny;
+    Q.N = Q.plane * I.nz;
+    Q.Ws = I.Ws; Q.Hs = I.Hs;
+    Q.Rs = kSlots * I.Ws;
+    Q.splane = Q.Rs * I.Hs;
+    Q.Ns = I.Ws;
+    Q.Nidx = Q.splane * I.nz - (kSlots - 1) * I.Ws;
+    Q.inv_N = I.inv_N;
+    Q.hot_cx = 0.5f * (float)I.nx;
+    Q.hot_cy = 0.5f * (float)I.ny;
+    return Q;
+}
+
 // Many independent lattices in one launch.  Persistent CTAs draw (instance, tile column) items
 // from a table through an atomic work counter, so uneven instances balance themselves; every
 // item runs the generic fused update above with the geometry of its instance and the shared
@@ -308,18 +328,7 @@ k_fused_batch(DevParams P, const BatchInst* __restrict__ insts, const BatchItem*
         if (it >= n_items) break;
         const BatchItem w = items[it];
         const BatchInst I = insts[w.inst];
-        DevParams Q = P;
-        Q.nx = I.nx; Q.ny = I.ny; Q.nz = I.nz;
-        Q.plane = I.nx * I.ny;
-        Q.N = Q.plane * I.nz;
-        Q.Ws = I.Ws; Q.Hs = I.Hs;
-        Q.Rs = kSlots * I.Ws;
-        Q.splane = Q.Rs * I.Hs;
-        Q.Ns = I.Ws;
-        Q.Nidx = Q.splane * I.nz - (kSlots - 1) * I.Ws;
-        Q.inv_N = I.inv_N;
-        Q.hot_cx = 0.5f * (float)I.nx;
-        Q.hot_cy = 0.5f * (float)I.ny;
+        const DevParams Q = instance_params(P, I);
         float r_sum = 0.f, r_c = 0.f, t_sum = 0.f, t_c = 0.f;
         const float rho_ave = buoyancy_ref(P, sums_cur[2 * w.inst], I.inv_N);
         fused_column<S, TY, false>(Q, src + I.pop_off, dst + I.pop_off, pull_f, pull_g, rho_ave, phis + I.field_off, first,
@@ -350,6 +359,103 @@ k_fused_batch(DevParams P, const BatchInst* __restrict__ insts, const BatchItem*
         counters[0] = 0u;
         counters[1] = 0u;
     }
+}
+
+// ================================================================ read-out
+// Macroscopic fields in one pass over the populations: a block marches a 32 x 8 tile through a chunk
+// of planes; every thread pulls its node (or a node of the ring around the tile), puts (psi, rho) into
+// a four-plane shared ring and keeps rho, T and the first moment of its node for one plane, until
+// the ring holds the plane above; then u = (sum e f + F/2) / rho with F from the ring stencil.
+// Populations are read once (the ring's from L2) in place of twice by a psi pass and a moments pass.
+// kBatch: block b of the grid is item b of an ensemble's read-out table, its fields at field_off.
+template <typename S, int QT, bool kBatch>
+__global__ void __launch_bounds__(FusedShape<kTY, QT>::kThreads, 2)
+k_readout(DevParams P0, const BatchInst* __restrict__ insts, const BatchItem* __restrict__ items,
+          const S* __restrict__ src0, int pull_f, int pull_g, const double* __restrict__ sums_cur, int zchunk,
+          float* __restrict__ orho, float* __restrict__ oux, float* __restrict__ ouy, float* __restrict__ ouz,
+          float* __restrict__ oT, int* flag) {
+    using Sh = FusedShape<kTY, QT>;
+    __shared__ float2 ring[Sh::kRing * Sh::kRingPlane];
+    int x0, y0, z0, z1, inst = 0;
+    long long pop_off = 0, field_off = 0;
+    DevParams Pi;
+    if constexpr (kBatch) {
+        const BatchItem w = items[blockIdx.x];
+        const BatchInst I = insts[w.inst];
+        Pi = instance_params(P0, I);
+        inst = w.inst;
+        pop_off = I.pop_off;
+        field_off = I.field_off;
+        x0 = w.x0; y0 = w.y0; z0 = w.z0; z1 = w.z1;
+    } else {
+        x0 = blockIdx.x * TX;
+        y0 = blockIdx.y * kTY;
+        z0 = blockIdx.z * zchunk;
+        z1 = min(P0.nz, z0 + zchunk);
+    }
+    const DevParams& P = kBatch ? Pi : P0;
+    const S* __restrict__ src = src0 + pop_off;
+    int lx, ly;
+    slot_of<kTY>(threadIdx.x, lx, ly);
+    const int gx = x0 + lx - 1, gy = y0 + ly - 1;
+    const bool slot_used = lx >= 0 && gx >= -1 && gx <= P.nx && gy >= -1 && gy <= P.ny;
+    const int mx = slot_used ? map_coord(gx, P.nx, P.bc[0], P.bc[1]) : 0;
+    const int my = slot_used ? map_coord(gy, P.ny, P.bc[2], P.bc[3]) : 0;
+    const bool owner = threadIdx.x < Sh::kInterior && gx < P.nx && gy < P.ny;
+    const int slot = slot_used ? bbase(P, ly * Sh::kRingW + lx, 0, 0, Sh::kRingPlane) : 0;
+    const float rho_ave = buoyancy_ref(P, sums_cur[2 * inst], P.inv_N);
+    struct Node {
+        float psi, rho, T, jx, jy, jz;
+    };
+    int bad = 0;
+    auto psi_pass = [&](int zp, Node& o) {
+        if (!slot_used) return;
+        float2* rp = ring + ((zp + 4) % Sh::kRing) * Sh::kRingPlane + slot;
+        if (!kBatch && zp < 0 && P.wet) {   // solid layer below a wetting -z wall: virtual (psi, rho)
+            *rp = wall_entry(P, mx, my);
+            return;
+        }
+        const int mz = map_coord(zp, P.nz, P.bc[4], P.bc[5]);
+        const int i = sidx(P, mx, my, mz);
+        const Nbr n = make_nbr(P, mx, my, mz);
+        float f[19], g[QT];
+        load_f<S>(P, src, pull_f, i, mx, my, mz, n, f);
+        Therm<QT>::template load<S>(P, src, pull_g, i, mx, my, mz, n, g);
+        o.rho = sum19(f);
+        o.T = Therm<QT>::sum(g);
+        const float psi2 = psi_squared(P, o.rho, o.T);
+        o.psi = psi_of(psi2);
+        *rp = make_float2(o.psi, o.rho);
+        bad |= !(psi2 > 0.f) || !isfinite(o.rho) || !isfinite(o.T);
+        o.jx = (f[1] - f[2]) + (f[7] - f[8]) + (f[9] - f[10]) + (f[11] - f[12]) + (f[13] - f[14]);
+        o.jy = (f[3] - f[4]) + (f[7] - f[8]) - (f[9] - f[10]) + (f[15] - f[16]) + (f[17] - f[18]);
+        o.jz = (f[5] - f[6]) + (f[11] - f[12]) - (f[13] - f[14]) + (f[15] - f[16]) - (f[17] - f[18]);
+    };
+    Node cur = {}, above = {};
+    psi_pass(z0 - 1, above);
+    psi_pass(z0, cur);
+    for (int z = z0; z < z1; ++z) {
+        psi_pass(z + 1, above);
+        __syncthreads();
+        if (owner) {
+            const RingStencil rs = ring_stencil(ring + ((z + 3) % Sh::kRing) * Sh::kRingPlane, ring + (z % Sh::kRing) * Sh::kRingPlane,
+                                                ring + ((z + 1) % Sh::kRing) * Sh::kRingPlane,
+                                                bbase(P, slot, -(Sh::kRingW + 1), Sh::kRingW + 1, Sh::kRingPlane), Sh::kRingW);
+            const float db = cur.rho - rho_ave;
+            const float Fx = __fmaf_rn(cur.psi, rs.Fx, __fmul_rn(db, P.gx)), Fy = __fmaf_rn(cur.psi, rs.Fy, __fmul_rn(db, P.gy)),
+                        Fz = __fmaf_rn(cur.psi, rs.Fz, __fmul_rn(db, P.gz));
+            const float inv = 1.f / cur.rho;
+            const bool fz = P.flow_off != 0;
+            const long long d = field_off + bidx(P, node_of(P, gx, gy, z), P.N);
+            if (orho) orho[d] = cur.rho;
+            if (oux) oux[d] = fz ? 0.f : (cur.jx + 0.5f * Fx) * inv;
+            if (ouy) ouy[d] = fz ? 0.f : (cur.jy + 0.5f * Fy) * inv;
+            if (ouz) ouz[d] = fz ? 0.f : (cur.jz + 0.5f * Fz) * inv;
+            if (oT) oT[d] = cur.T;
+        }
+        cur = above;
+    }
+    if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(flag, 1);
 }
 
 // ================================================================ TMA producer / consumer kernel
@@ -1259,6 +1365,53 @@ cudaError_t launch_fused(const DevParams& P, int precision, const StateBufs& B, 
     }
 #undef GB300_FUSED
     if (e != cudaSuccess) return e;
+    return cudaGetLastError();
+}
+
+// planes of a read-out block: about six blocks for each of the two resident on an SM, so that the
+// last wave is short, at least two planes (a block reads two more than it writes)
+static int zchunk_readout(const DevParams& P, long long tiles) {
+    const long long target = (long long)device_sms() * 12;
+    const int chunks = (int)std::max<long long>(1, std::min<long long>(target / tiles, P.nz / 2));
+    return (P.nz + chunks - 1) / chunks;
+}
+
+cudaError_t launch_readout(const DevParams& P, int precision, const StateBufs& B, const double* sums_cur, float* rho,
+                           float* ux, float* uy, float* uz, float* T, cudaStream_t s) {
+    const int tiles_x = (P.nx + TX - 1) / TX, tiles_y = (P.ny + kTY - 1) / kTY;
+    const int zc = zchunk_readout(P, (long long)tiles_x * tiles_y);
+    const dim3 grid(tiles_x, tiles_y, (P.nz + zc - 1) / zc);
+#define GB300_READ(S, QT)                                                                                      \
+    k_readout<S, QT, false><<<grid, FusedShape<kTY, QT>::kThreads, 0, s>>>(P, nullptr, nullptr, (const S*)B.src, \
+                                                                           B.pull_f, B.pull_g, sums_cur, zc, rho, ux, uy, uz, T, B.flag)
+    if (P.qt == 19) {
+        if (precision != 0) return cudaErrorInvalidValue;
+        GB300_READ(float, 19);
+    } else {
+        switch (precision) {
+        case 0: GB300_READ(float, 7); break;
+        case 1: GB300_READ(__nv_bfloat16, 7); break;
+        case 2: GB300_READ(__half, 7); break;
+        default: return cudaErrorInvalidValue;
+        }
+    }
+#undef GB300_READ
+    return cudaGetLastError();
+}
+
+cudaError_t launch_readout_batch(const DevParams& P, int precision, const BatchInst* insts, const BatchItem* items,
+                                 int n_items, const StateBufs& B, const double* sums_cur, float* rho, float* ux,
+                                 float* uy, float* uz, float* T, cudaStream_t s) {
+#define GB300_READ(S)                                                                                          \
+    k_readout<S, 7, true><<<n_items, FusedShape<kTY>::kThreads, 0, s>>>(P, insts, items, (const S*)B.src, B.pull_f, \
+                                                                        B.pull_g, sums_cur, 0, rho, ux, uy, uz, T, B.flag)
+    switch (precision) {
+    case 0: GB300_READ(float); break;
+    case 1: GB300_READ(__nv_bfloat16); break;
+    case 2: GB300_READ(__half); break;
+    default: return cudaErrorInvalidValue;
+    }
+#undef GB300_READ
     return cudaGetLastError();
 }
 

@@ -226,38 +226,6 @@ __global__ void __launch_bounds__(TPB) k_collide(DevParams P, const S* __restric
     phis[d] = ph;
 }
 
-// ---------------------------------------------------------------- moments (lbm_get_moments)
-template <typename S, int QT>
-__global__ void __launch_bounds__(TPB) k_moments(DevParams P, const S* __restrict__ fs, int pull_f, int pull_g, const float2* __restrict__ psirho,
-                                                const double* __restrict__ sums_cur, float* __restrict__ orho,
-                                                float* __restrict__ oux, float* __restrict__ ouy,
-                                                float* __restrict__ ouz, float* __restrict__ oT) {
-    int x = blockIdx.x * TPB_X + threadIdx.x, y = blockIdx.y * TPB_Y + threadIdx.y, z = blockIdx.z;
-    if (x >= P.nx || y >= P.ny) return;
-    int i = sidx(P, x, y, z);
-    Nbr n = make_nbr(P, x, y, z);
-    float f[19], g[QT];
-    load_f<S>(P, fs, pull_f, i, x, y, z, n, f);
-    Therm<QT>::template load<S>(P, fs, pull_g, i, x, y, z, n, g);
-    float rho = sum19(f), T = Therm<QT>::sum(g);
-    i = node_of(P, x, y, z);
-    float jx = (f[1] - f[2]) + (f[7] - f[8]) + (f[9] - f[10]) + (f[11] - f[12]) + (f[13] - f[14]);
-    float jy = (f[3] - f[4]) + (f[7] - f[8]) - (f[9] - f[10]) + (f[15] - f[16]) + (f[17] - f[18]);
-    float jz = (f[5] - f[6]) + (f[11] - f[12]) - (f[13] - f[14]) + (f[15] - f[16]) - (f[17] - f[18]);
-    float2 me = __ldg(psirho + i);
-    Stencil st = stencil(P, psirho, x, y, z, n);
-    float rho_ave = buoyancy_ref(P, sums_cur[0], P.inv_N);
-    float db = rho - rho_ave;
-    float Fx = me.x * st.x.x + db * P.gx, Fy = me.x * st.y.x + db * P.gy, Fz = me.x * st.z.x + db * P.gz;
-    float inv = 1.f / rho;
-    bool fz = P.flow_off != 0;
-    if (orho) orho[i] = rho;
-    if (oux) oux[i] = fz ? 0.f : (jx + 0.5f * Fx) * inv;
-    if (ouy) ouy[i] = fz ? 0.f : (jy + 0.5f * Fy) * inv;
-    if (ouz) ouz[i] = fz ? 0.f : (jz + 0.5f * Fz) * inv;
-    if (oT) oT[i] = T;
-}
-
 // ---------------------------------------------------------------- field sum
 __global__ void __launch_bounds__(256) k_sum_field(const float* __restrict__ a, int n, double2* partial,
                                                    unsigned* counter, double* out) {
@@ -395,14 +363,6 @@ cudaError_t launch_velocity(const DevParams& P, int precision, const StateBufs& 
     dim3 blk(TPB_X, TPB_Y);
     GB300_DISPATCH(precision, (k_velocity<S><<<grid_of(P), blk, 0, s>>>(P, (const S*)B.src, B.pull_f, B.psirho,
                                                                          sums_cur, B.vel)));
-    return cudaGetLastError();
-}
-
-cudaError_t launch_moments(const DevParams& P, int precision, const StateBufs& B, const double* sums_cur,
-                           float* rho, float* ux, float* uy, float* uz, float* T, cudaStream_t s) {
-    dim3 blk(TPB_X, TPB_Y);
-    GB300_DISPATCH_QT(P, precision, (k_moments<S, QT><<<grid_of(P), blk, 0, s>>>(P, (const S*)B.src, B.pull_f, B.pull_g,
-                                                                        B.psirho, sums_cur, rho, ux, uy, uz, T)));
     return cudaGetLastError();
 }
 

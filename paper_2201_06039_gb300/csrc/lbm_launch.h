@@ -101,10 +101,10 @@ int tma_ghost_mode(const DevParams& P, int shape, int precision);
 int tma_ghost_cols(int precision);
 int tma_tile_h(int shape);
 
-// macroscopic moments (needs the psi pass on the same state first).
-cudaError_t launch_moments(const DevParams& P, int precision, const StateBufs& B,
-                           const double* sums_cur, float* rho, float* ux, float* uy, float* uz,
-                           float* T, cudaStream_t s);
+// macroscopic fields of the current state (B.src) into the device arrays given (each nullable); a
+// scheme-1 wetting wall's table must be that of this state
+cudaError_t launch_readout(const DevParams& P, int precision, const StateBufs& B, const double* sums_cur, float* rho,
+                           float* ux, float* uy, float* uz, float* T, cudaStream_t s);
 
 // deterministic FP64 sum of a float field into out[0] (out[1] = 0).
 cudaError_t launch_sum_field(const float* a, int n, double2* partial, unsigned* counter,
@@ -132,6 +132,11 @@ struct BatchItem {
 cudaError_t launch_fused_batch(const DevParams& P, int precision, int ty, const BatchInst* insts,
                                const BatchItem* items, int n_items, int n_inst, const StateBufs& B,
                                const double* sums_cur, double* sums_next, int first, int ctas, cudaStream_t s);
+// macroscopic fields of every instance in one launch: items are 32 x 8 tiles (x0, y0) and planes [z0, z1)
+// of the instances, any order, each node in one item; outputs concatenated in instance order
+cudaError_t launch_readout_batch(const DevParams& P, int precision, const BatchInst* insts, const BatchItem* items,
+                                 int n_items, const StateBufs& B, const double* sums_cur, float* rho, float* ux,
+                                 float* uy, float* uz, float* T, cudaStream_t s);
 // resident CTAs per SM of the batched kernel (0 if it cannot launch)
 int batch_ctas_per_sm(int precision, int ty);
 int batch_tile_rows(int ty);
