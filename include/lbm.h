@@ -65,8 +65,8 @@ typedef enum {
     LBM_KERNEL_TWO_PASS = 1,  /* psi/EOS kernel, then the stream-collide kernel */
     LBM_KERNEL_FUSED = 2,     /* one z-marching kernel per step (halo recomputation) */
     LBM_KERNEL_FUSED_TMA = 3  /* reported by lbm_kernel_in_use: FUSED with TMA-fed pipeline (any
-                                 storage precision; x and y faces periodic or thermal-only;
-                                 nx, ny >= 4; flow and temperature both evolving) */
+                                 storage precision and faces; nx, ny >= 4; flow evolving; a frozen
+                                 temperature or a wetting wall with FP32 storage) */
 } lbm_kernel_variant;
 
 typedef struct {
@@ -204,11 +204,11 @@ int lbm_load_state(lbm_ctx* ctx, const void* buf, size_t bytes);
 int lbm_set_wall_map(lbm_ctx* ctx, const float* phi, const float* drho);
 
 /* Kernel variant the context runs (LBM_KERNEL_TWO_PASS, LBM_KERNEL_FUSED or
- * LBM_KERNEL_FUSED_TMA; AUTO resolved).  The first step after lbm_init_fields, and steps with a
- * frozen field, always run the generic fused kernel. */
+ * LBM_KERNEL_FUSED_TMA; AUTO resolved).  The first step after lbm_init_fields always runs the
+ * generic fused kernel. */
 int lbm_kernel_in_use(const lbm_ctx* ctx);
 
-/* Tile plan of the TMA kernel (the default path on lattices with f-periodic x and y faces).  A
+/* Tile plan of the TMA kernel (the default path; see LBM_KERNEL_FUSED_TMA for what it covers).  A
  * persistent CTA per SM marches tiles of tile_w x tile_h nodes up z; the lattice is cut into
  * items (tile, z-chunk of zchunk planes) taken round robin by the CTAs.  The plan is chosen at
  * lbm_create from a model of the kernel's cost; these calls report, pin or measure it.  Plans do

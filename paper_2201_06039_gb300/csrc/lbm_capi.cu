@@ -195,6 +195,11 @@ DevParams make_dev(const lbm_params* p) {
     d.Ns = d.Ws;
     d.Nidx = d.splane * p->nz - (slots - 1) * d.Ws;
     for (int k = 0; k < 6; ++k) { d.bc[k] = p->bc[k]; d.T_wall[k] = (float)p->T_wall[k]; }
+    for (int k = 0; k < 4; ++k) {
+        if (d.bc[k] != BC_PERIODIC) d.xy_faces |= 1u << k;
+        if (d.bc[k] == BC_WALL) d.xy_walls |= 1u << k;
+        if (d.bc[k] == BC_OUTFLOW) d.xy_open |= 1u << k;
+    }
     d.hot_dT = (float)p->hot_dT;
     d.hot_inv2s2 = p->hot_dT != 0.0 ? (float)(1.0 / (2.0 * p->hot_sigma * p->hot_sigma)) : 0.f;
     d.hot_cx = 0.5f * (float)p->nx;
@@ -324,7 +329,7 @@ int enqueue_step(lbm_ctx* c, KernelTimer* timer = nullptr) {
         e = launch_fused(c->dp, c->p.precision, B, c->sums(c->slot), c->sums(c->slot ^ 1), c->first ? 1 : 0,
                          c->launch, c->maps.ok ? &c->maps : nullptr, &ghosts_done);
         if (e != cudaSuccess) return fail(LBM_ECUDA, "fused kernel launch: %s", cudaGetErrorString(e));
-        if (c->maps.ok && B.pull_f && B.pull_g) c->dp.test_stall = 0;   // one stalled TMA step only
+        if (c->maps.ok && tma_runs(c->dp, c->p.precision, B)) c->dp.test_stall = 0;   // one stalled TMA step only
         if (timer) timer->end(0, c->launch);
     } else {
         if (timer) timer->begin(c->launch);
@@ -808,7 +813,7 @@ int lbm_load_state(lbm_ctx* c, const void* buf, size_t bytes) {
     CK(cudaMemcpyAsync(c->sums(c->slot), in + h.pop_bytes + h.phis_bytes, 2 * sizeof(double), cudaMemcpyHostToDevice,
                        c->stream));
     // the saving context may not have kept the ghost cells (kernels without TMA do not use them)
-    if (c->maps.ok && !h.fresh_f && !h.fresh_g) CK(launch_ghosts(c->dp, c->p.precision, c->pbuf(c->cur), c->stream));
+    if (c->maps.ok && !(h.fresh_f && h.fresh_g)) CK(launch_ghosts(c->dp, c->p.precision, c->pbuf(c->cur), c->stream));
     CK(cudaMemsetAsync(c->base + c->L.flag, 0, sizeof(int), c->stream));
     CK(cudaStreamSynchronize(c->stream));
     c->fresh_f = h.fresh_f != 0;
@@ -867,7 +872,7 @@ int lbm_autotune(lbm_ctx* c, int steps, double* best_ms) {
         return fail(LBM_ESTATE, "the context does not run the TMA kernel");
     // the first step after lbm_init_fields runs the generic kernel: take it before timing
     int rc = LBM_OK;
-    while (rc == LBM_OK && (c->first || c->fresh_f || c->fresh_g)) rc = enqueue_step(c);
+    while (rc == LBM_OK && (c->first || (c->fresh_f && !c->p.flow_off) || (c->fresh_g && !c->p.thermal_off))) rc = enqueue_step(c);
     if (rc) return rc;
     const size_t popb = pop_elems(c->dp) * pop_bytes(c->p.precision), phib = 4 * (size_t)c->dp.N;
     const size_t sumb = 8 * sizeof(double);

@@ -92,6 +92,7 @@ struct DevParams {
     float shift_g[7];         // storage shift w_a T_ref
     int* check_flag;          // the context's flag word (bounds-checked builds record violations here)
     int qt;                   // temperature lattice: 7 (D3Q7 MRT) or 19 (Eq. 19 BGK on D3Q19)
+    unsigned xy_faces, xy_walls, xy_open;   // x and y faces (bits -x, +x, -y, +y) not periodic for g / wall / outflow
 };
 
 // Debug builds (-DLBM_BOUNDS_CHECK): every population and field index of the update, and the

@@ -13,8 +13,8 @@
 // the buoyancy force is the deterministic FP64 mean of this step's rho, used by the next step.
 //
 // k_fused     : generic (any faces, any storage precision, frozen f or g, first step).
-// k_fused_tma : FP32 or shifted 16-bit storage, f-periodic x and y faces (any z faces).  A
-//               producer warp fetches each plane's pulls for the whole tile + halo with three TMA
+// k_fused_tma : FP32 or shifted 16-bit storage, any faces, g evolving (or frozen, FP32).  A
+//               copy warp fetches each plane's pulls for the whole tile + halo with three TMA
 //               tensor copies (one per e_z group of population slots) into a multi-stage
 //               shared-memory pipeline guarded by mbarriers; psi warps and collision warps read
 //               every pull as one shared-memory load at a fixed offset.  FP32 planes leave through
@@ -23,6 +23,7 @@
 #include <cuda.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "lbm_launch.h"
 
@@ -642,13 +643,46 @@ template <> __device__ __forceinline__ __nv_bfloat16 st_enc<__nv_bfloat16>(float
 }
 template <> __device__ __forceinline__ __half st_enc<__half>(float v, float sh) { return __float2half_rn(v - sh); }
 
+// Faces across x and y.  Where f does not wrap, the nodes of the face column or row have their crossing
+// links patched, in place of leaving such lattices to the generic kernel: a closed box of 150 x 110 x 130
+// 169 -> 128 us a step; with a frozen g, a sessile drop of 200 x 200 x 100 270 -> 218.
+//
+// f_A of a node at outflow faces of x or y (bits -x, +x, -y, +y of open): the clamped source; links that
+// cross a z wall (bits 16, 32 of z_walls) are bounced back already.
+template <class Sh, int A>
+__device__ __forceinline__ void patch_open(const DevParams& P, const typename Sh::S* __restrict__ b, unsigned open,
+                                           unsigned z_walls, float f[19]) {
+    using S = typename Sh::S;
+    constexpr int ex = ex19(A), ey = ey19(A), ez = ez19(A);
+    constexpr unsigned mx = ex > 0 ? 1u : ex < 0 ? 2u : 0u, my = ey > 0 ? 4u : ey < 0 ? 8u : 0u;
+    constexpr unsigned mz = ez > 0 ? 16u : ez < 0 ? 32u : 0u;
+    if ((open & (mx | my)) && !(z_walls & mz))
+        f[A] = st_dec<S>(b[Sh::slot_off(fslot(A)) - (open & my ? 0 : ey * Sh::kWinW) - (open & mx ? 0 : ex)], P.shift_f[A]);
+}
+// f_A of a node at an x or y wall that the link crosses: f*_abar of the node itself (Eq. 50), from the
+// stage, or from global memory where the stage holds another plane of that slot.
+template <class Sh, int A>
+__device__ __forceinline__ void patch_wall(const DevParams& P, const typename Sh::S* __restrict__ b,
+                                           const typename Sh::S* __restrict__ src, int i, float f[19]) {
+    using S = typename Sh::S;
+    f[A] = ez19(A) == 0 ? st_dec<S>(b[Sh::slot_off(fslot(opp(A)))], P.shift_f[opp(A)])
+                        : Codec<S>::load(src + (size_t)fslot(opp(A)) * P.Ns + i, P.shift_f[opp(A)]);
+}
+
+// the x and y faces not periodic for g that (mx, my) lies at (bits -x, +x, -y, +y)
+__device__ __forceinline__ unsigned faces_at(const DevParams& P, int mx, int my) {
+    return P.xy_faces & ((mx == 0 ? 1u : 0u) | (mx == P.nx - 1 ? 2u : 0u) | (my == 0 ? 4u : 0u) | (my == P.ny - 1 ? 8u : 0u));
+}
+
 // The 26 pulled populations of the node whose window cell is b (a pointer into a stage), with the
 // boundary links of its plane mz patched: Eq. 50 for f at z walls (f*_abar of the node itself,
 // read from global memory), Eq. 51 for g at non-periodic z faces (own g+_abar from global memory)
-// and at thermal x / y faces (own g+_abar from the stage).
-template <class Sh>
+// and at x / y faces (own g+_abar from the stage), Eq. 50 or the clamped source for f at x / y walls
+// and outflow faces (at: faces_at of the node).  kFrozen: g is the node's own stored g (it does not
+// stream).
+template <class Sh, bool kFrozen>
 __device__ __forceinline__ void stage_pulls(const DevParams& P, const typename Sh::S* __restrict__ b,
-                                            const typename Sh::S* __restrict__ src, int mx, int my, int mz,
+                                            const typename Sh::S* __restrict__ src, int mx, int my, int mz, unsigned at,
                                             float f[19], float g[7]) {
     using S = typename Sh::S;
     constexpr int WW = Sh::kWinW;
@@ -657,9 +691,17 @@ __device__ __forceinline__ void stage_pulls(const DevParams& P, const typename S
     GB300_SF(9) GB300_SF(10) GB300_SF(11) GB300_SF(12) GB300_SF(13) GB300_SF(14) GB300_SF(15) GB300_SF(16)
     GB300_SF(17) GB300_SF(18)
 #undef GB300_SF
+    if constexpr (kFrozen) {
+        const int i = (int)bidx(P, sidx(P, mx, my, mz), P.Nidx);
+#pragma unroll
+        for (int a = 0; a < 5; ++a) g[a] = st_dec<S>(b[Sh::slot_off(gslot(a))], P.shift_g[a]);
+        g[5] = Codec<S>::load(src + (size_t)gslot(5) * P.Ns + i, P.shift_g[5]);   // the stage holds these of planes
+        g[6] = Codec<S>::load(src + (size_t)gslot(6) * P.Ns + i, P.shift_g[6]);   // z - 1 and z + 1
+    } else {
 #define GB300_SG(A) g[A] = st_dec<S>(b[Sh::slot_off(gslot(A)) - ey7(A) * WW - ex7(A)], P.shift_g[A]);
-    GB300_SG(0) GB300_SG(1) GB300_SG(2) GB300_SG(3) GB300_SG(4) GB300_SG(5) GB300_SG(6)
+        GB300_SG(0) GB300_SG(1) GB300_SG(2) GB300_SG(3) GB300_SG(4) GB300_SG(5) GB300_SG(6)
 #undef GB300_SG
+    }
     if (mz == 0 && P.bc[4] != BC_PERIODIC) {
         const int i = (int)bidx(P, sidx(P, mx, my, mz), P.Nidx);
         if (P.bc[4] == BC_WALL) {
@@ -669,7 +711,8 @@ __device__ __forceinline__ void stage_pulls(const DevParams& P, const typename S
             f[15] = Codec<S>::load(src + (size_t)fslot(16) * P.Ns + i, P.shift_f[16]);
             f[18] = Codec<S>::load(src + (size_t)fslot(17) * P.Ns + i, P.shift_f[17]);
         }
-        g[5] = -Codec<S>::load(src + (size_t)gslot(6) * P.Ns + i, P.shift_g[6]) + 2.f * P.w1 * wall_T(P, 4, mx, my);
+        if (!kFrozen)
+            g[5] = -Codec<S>::load(src + (size_t)gslot(6) * P.Ns + i, P.shift_g[6]) + 2.f * P.w1 * wall_T(P, 4, mx, my);
     }
     if (mz == P.nz - 1 && P.bc[5] != BC_PERIODIC) {
         const int i = (int)bidx(P, sidx(P, mx, my, mz), P.Nidx);
@@ -680,16 +723,36 @@ __device__ __forceinline__ void stage_pulls(const DevParams& P, const typename S
             f[16] = Codec<S>::load(src + (size_t)fslot(15) * P.Ns + i, P.shift_f[15]);
             f[17] = Codec<S>::load(src + (size_t)fslot(18) * P.Ns + i, P.shift_f[18]);
         }
-        g[6] = -Codec<S>::load(src + (size_t)gslot(5) * P.Ns + i, P.shift_g[5]) + 2.f * P.w1 * wall_T(P, 5, mx, my);
+        if (!kFrozen)
+            g[6] = -Codec<S>::load(src + (size_t)gslot(5) * P.Ns + i, P.shift_g[5]) + 2.f * P.w1 * wall_T(P, 5, mx, my);
     }
-    if (P.bc[0] == BC_THERMAL_ONLY && mx == 0)
-        g[1] = -st_dec<S>(b[Sh::slot_off(gslot(2))], P.shift_g[2]) + 2.f * P.w1 * wall_T(P, 0, mx, my);
-    if (P.bc[1] == BC_THERMAL_ONLY && mx == P.nx - 1)
-        g[2] = -st_dec<S>(b[Sh::slot_off(gslot(1))], P.shift_g[1]) + 2.f * P.w1 * wall_T(P, 1, mx, my);
-    if (P.bc[2] == BC_THERMAL_ONLY && my == 0)
-        g[3] = -st_dec<S>(b[Sh::slot_off(gslot(4))], P.shift_g[4]) + 2.f * P.w1 * wall_T(P, 2, mx, my);
-    if (P.bc[3] == BC_THERMAL_ONLY && my == P.ny - 1)
-        g[4] = -st_dec<S>(b[Sh::slot_off(gslot(3))], P.shift_g[3]) + 2.f * P.w1 * wall_T(P, 3, mx, my);
+    if (P.xy_faces) {   // uniform: some x or y face is not periodic
+        if (!kFrozen) {
+            if (at & 1u) g[1] = -st_dec<S>(b[Sh::slot_off(gslot(2))], P.shift_g[2]) + 2.f * P.w1 * wall_T(P, 0, mx, my);
+            if (at & 2u) g[2] = -st_dec<S>(b[Sh::slot_off(gslot(1))], P.shift_g[1]) + 2.f * P.w1 * wall_T(P, 1, mx, my);
+            if (at & 4u) g[3] = -st_dec<S>(b[Sh::slot_off(gslot(4))], P.shift_g[4]) + 2.f * P.w1 * wall_T(P, 2, mx, my);
+            if (at & 8u) g[4] = -st_dec<S>(b[Sh::slot_off(gslot(3))], P.shift_g[3]) + 2.f * P.w1 * wall_T(P, 3, mx, my);
+        }
+        if ((P.xy_open | P.xy_walls) == 0u) return;   // uniform: g only
+        if (at & P.xy_open) {
+            const unsigned open = at & P.xy_open, z_walls = (mz == 0 && P.bc[4] == BC_WALL ? 16u : 0u) |
+                                                            (mz == P.nz - 1 && P.bc[5] == BC_WALL ? 32u : 0u);
+#define GB300_PF(A) patch_open<Sh, A>(P, b, open, z_walls, f);
+            GB300_PF(1) GB300_PF(2) GB300_PF(3) GB300_PF(4) GB300_PF(7) GB300_PF(8) GB300_PF(9) GB300_PF(10)
+            GB300_PF(11) GB300_PF(12) GB300_PF(13) GB300_PF(14) GB300_PF(15) GB300_PF(16) GB300_PF(17) GB300_PF(18)
+#undef GB300_PF
+        }
+        if (at & P.xy_walls) {   // after the outflow faces: a link that crosses both bounces back
+            const unsigned walls = at & P.xy_walls;
+            const int i = (int)bidx(P, sidx(P, mx, my, mz), P.Nidx);
+#define GB300_PW(A) patch_wall<Sh, A>(P, b, src, i, f);
+            if (walls & 1u) { GB300_PW(1) GB300_PW(7) GB300_PW(9) GB300_PW(11) GB300_PW(13) }
+            if (walls & 2u) { GB300_PW(2) GB300_PW(8) GB300_PW(10) GB300_PW(12) GB300_PW(14) }
+            if (walls & 4u) { GB300_PW(3) GB300_PW(7) GB300_PW(10) GB300_PW(15) GB300_PW(17) }
+            if (walls & 8u) { GB300_PW(4) GB300_PW(8) GB300_PW(9) GB300_PW(16) GB300_PW(18) }
+#undef GB300_PW
+        }
+    }
 }
 
 // named barriers of the TMA kernel (bar.sync / bar.arrive; 0 is __syncthreads): the waiting
@@ -727,7 +790,7 @@ __device__ __forceinline__ void nb_arrive(int id, int nthreads) {
 // halo); the copy warp's next arrival on RING(s) follows its OUT_FULL(s) sync of the previous use of
 // s, whose arrivals follow that use's RING(s); and the compute warps' next arrival on OUT_FULL(s)
 // follows their RING(s) sync of the next use of s, which needs that arrival of the copy warp.
-template <int TX_, int TY_, typename S, bool kWet>
+template <int TX_, int TY_, typename S, bool kWet, bool kFrozen>
 __global__ void __maxnreg__((TmaShape<TX_, TY_, S>::kMaxRegs))
 k_fused_tma(const __grid_constant__ CUtensorMap map14, const __grid_constant__ CUtensorMap map6,
             const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_out_top,
@@ -896,6 +959,9 @@ k_fused_tma(const __grid_constant__ CUtensorMap map14, const __grid_constant__ C
             const bool used = node_thread && gx <= P.nx && gy <= P.ny;
             const int mx = used ? map_coord(gx, P.nx, P.bc[0], P.bc[1]) : 0;
             const int my = used ? map_coord(gy, P.ny, P.bc[2], P.bc[3]) : 0;
+            const unsigned at = used ? faces_at(P, mx, my) : 0u;
+            // its window cell: the image's own, or the mirror node's past a face that f does not wrap
+            const int cell = woff - (gx == P.nx && !f_wraps(P.bc[1]) ? 1 : 0) - (gy == P.ny && !f_wraps(P.bc[3]) ? kWinW : 0);
             // this node's place in the ghost staging tiles of an edge tile (-1: none)
             const bool eright = ghosts == 1 && x0 + TX_ >= P.nx, eleft = ghosts == 1 && x0 == 0;
             const bool etop = ghosts == 1 && y0 + TY_ >= P.ny, ebottom = ghosts == 1 && y0 == 0;
@@ -924,7 +990,7 @@ k_fused_tma(const __grid_constant__ CUtensorMap map14, const __grid_constant__ C
                     if (used) *rp = wall_entry(P, mx, my);
                 } else if (used) {
                     const int mz = map_coord(p, P.nz, P.bc[4], P.bc[5]);
-                    stage_pulls<Sh>(P, stage_of(s) + woff, src, mx, my, mz, fo, go);
+                    stage_pulls<Sh, kFrozen>(P, stage_of(s) + cell, src, mx, my, mz, at, fo, go);
                     ro = sum19(fo);
                     To = sum7(go);
                     const float psi2 = psi_squared(P, ro, To);
@@ -943,8 +1009,43 @@ k_fused_tma(const __grid_constant__ CUtensorMap map14, const __grid_constant__ C
                 const int so = (k - 1) % kStages;       // the stage just pulled receives plane z
                 const float ph_prev = ph_next;
                 if (owner && z + 1 < z1) ph_next = phis[bidx(P, node_of(P, gx, gy, z + 1), P.N)];
+                // the stored form of the node's populations to the out tile, or straight to dst, and to the
+                // ghost cells that hold its images: f and g, or one of them (kF, kG)
+                auto store = [&](auto kF, auto kG) {
+                    S fe[19], ge[7];
+                    auto put = [&](S* q, size_t stride) {
+                        if constexpr (kF.value) {
+#pragma unroll
+                            for (int a = 0; a < 19; ++a) q[fslot(a) * stride] = fe[a];
+                        }
+                        if constexpr (kG.value) {
+#pragma unroll
+                            for (int a = 0; a < 7; ++a) q[gslot(a) * stride] = ge[a];
+                        }
+                    };
+#pragma unroll
+                    for (int a = 0; a < 19; ++a) fe[a] = st_enc<S>(fc[a], P.shift_f[a]);
+#pragma unroll
+                    for (int a = 0; a < 7; ++a) ge[a] = st_enc<S>(gc[a], P.shift_g[a]);
+                    S* const sb = reinterpret_cast<S*>(smem_raw + (size_t)so * Sh::kStageOne);
+                    if (direct_tile) put(dst + bidx(P, sidx(P, gx, gy, z), P.Nidx), P.Ns);
+                    else put(sb + ooff, TX_);
+                    if (cx4 >= 0)   // edge column: [TY][26][kGW]
+                        put(sb + Sh::kGColOff / sizeof(S) + (ly - 1) * (kSlots * kGW) + cx4, kGW);
+                    if (ry2 >= 0)   // edge row: [2][26][rw]
+                        put(sb + Sh::kGRowOff / sizeof(S) + ry2 * (kSlots * rw) + (lx - 1), rw);
+                    if (cx4 >= 0 && ry2 >= 0)   // corner block: [2][26][kGW]
+                        put(sb + Sh::kGCorOff / sizeof(S) + ry2 * (kSlots * kGW) + cx4, kGW);
+                    // ghost mode 2: straight to the images in dst
+                    if (hx) put(dst + bidx(P, sidx(P, ix, gy, z), P.Nidx), P.Ns);
+                    if (hy) put(dst + bidx(P, sidx(P, gx, iy, z), P.Nidx), P.Ns);
+                    if (hx && hy) put(dst + bidx(P, sidx(P, ix, iy, z), P.Nidx), P.Ns);
+                };
+                constexpr std::true_type yes{};
+                constexpr std::false_type no{};
                 float ph = 0.f;
                 if (owner) {
+                    if constexpr (kFrozen) store(no, yes);   // the pulled g is the stored one: it stays
                     const float2* rm = ring + ((k - 3) % kRing) * kRP;
                     const float2* r0 = ring + ((k - 2) % kRing) * kRP;
                     const float2* rq = ring + ((k - 1) % kRing) * kRP;
@@ -954,66 +1055,12 @@ k_fused_tma(const __grid_constant__ CUtensorMap map14, const __grid_constant__ C
                     const Forces F = total_force(P, pc, rs.Fx, rs.Fy, rs.Fz, rc - rho_ave);
                     NodeOut o = collide_f(P, fc, rc, F.Fx, F.Fy, F.Fz, F.Fm2, pc * pc);
                     ph = collide_g(P, gc, rc, Tc, o, rs.gx, rs.gy, rs.gz, ph_prev, first);
+                    if constexpr (kFrozen) store(yes, no);
+                    else store(yes, yes);
                 }
-                {
-                    S* const sb = reinterpret_cast<S*>(smem_raw + (size_t)so * Sh::kStageOne);
-                    S* const outp = sb + ooff;
-                    if (owner) {
-                        S fe[19], ge[7];
-#pragma unroll
-                        for (int a = 0; a < 19; ++a) fe[a] = st_enc<S>(fc[a], P.shift_f[a]);
-#pragma unroll
-                        for (int a = 0; a < 7; ++a) ge[a] = st_enc<S>(gc[a], P.shift_g[a]);
-                        if (direct_tile) {
-                            S* q = dst + bidx(P, sidx(P, gx, gy, z), P.Nidx);
-#pragma unroll
-                            for (int a = 0; a < 19; ++a) q[(size_t)fslot(a) * P.Ns] = fe[a];
-#pragma unroll
-                            for (int a = 0; a < 7; ++a) q[(size_t)gslot(a) * P.Ns] = ge[a];
-                        } else {
-#pragma unroll
-                            for (int a = 0; a < 19; ++a) outp[fslot(a) * TX_] = fe[a];
-#pragma unroll
-                            for (int a = 0; a < 7; ++a) outp[gslot(a) * TX_] = ge[a];
-                        }
-                        if (cx4 >= 0) {   // edge column: [TY][26][kGW]
-                            S* q = sb + Sh::kGColOff / sizeof(S) + (ly - 1) * (kSlots * kGW) + cx4;
-#pragma unroll
-                            for (int a = 0; a < 19; ++a) q[fslot(a) * kGW] = fe[a];
-#pragma unroll
-                            for (int a = 0; a < 7; ++a) q[gslot(a) * kGW] = ge[a];
-                        }
-                        if (ry2 >= 0) {   // edge row: [2][26][rw]
-                            S* q = sb + Sh::kGRowOff / sizeof(S) + ry2 * (kSlots * rw) + (lx - 1);
-#pragma unroll
-                            for (int a = 0; a < 19; ++a) q[fslot(a) * rw] = fe[a];
-#pragma unroll
-                            for (int a = 0; a < 7; ++a) q[gslot(a) * rw] = ge[a];
-                        }
-                        if (cx4 >= 0 && ry2 >= 0) {   // corner block: [2][26][kGW]
-                            S* q = sb + Sh::kGCorOff / sizeof(S) + ry2 * (kSlots * kGW) + cx4;
-#pragma unroll
-                            for (int a = 0; a < 19; ++a) q[fslot(a) * kGW] = fe[a];
-#pragma unroll
-                            for (int a = 0; a < 7; ++a) q[gslot(a) * kGW] = ge[a];
-                        }
-                        if (hx || hy) {   // ghost mode 2: straight to the images in dst
-                            auto put = [&](int qx, int qy) {
-                                S* q = dst + bidx(P, sidx(P, qx, qy, z), P.Nidx);
-#pragma unroll
-                                for (int a = 0; a < 19; ++a) q[(size_t)fslot(a) * P.Ns] = fe[a];
-#pragma unroll
-                                for (int a = 0; a < 7; ++a) q[(size_t)gslot(a) * P.Ns] = ge[a];
-                            };
-                            if (hx) put(ix, gy);
-                            if (hy) put(gx, iy);
-                            if (hx && hy) put(ix, iy);
-                        }
-                    }
-                    // this thread's out writes become visible to the tensor store (async proxy)
-                    fence_proxy_async_smem();
-                    nb_arrive(bar_out_full(so), Sh::kCntOut);
-                }
+                // this thread's out writes become visible to the tensor store (async proxy)
+                fence_proxy_async_smem();
+                nb_arrive(bar_out_full(so), Sh::kCntOut);
                 if (owner) phis[bidx(P, node_of(P, gx, gy, z), P.N)] = ph;
             };
 
@@ -1056,14 +1103,18 @@ k_fused_tma(const __grid_constant__ CUtensorMap map14, const __grid_constant__ C
             const int z0 = chunk * zchunk, z1 = min(P.nz, z0 + zchunk);
             // per slot: lattice coordinates (-1: none), ring offset and window cell, once an item
             int mx[2], my[2], roff[2], woff[2];
+            unsigned at[2];
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
                 const int gx = x0 + lx[j] - 1, gy = y0 + ly[j] - 1;
                 const bool used = lx[j] >= 0 && gx <= P.nx && gy <= P.ny;
                 mx[j] = used ? map_coord(gx, P.nx, P.bc[0], P.bc[1]) : -1;
                 my[j] = used ? map_coord(gy, P.ny, P.bc[2], P.bc[3]) : 0;
+                at[j] = used ? faces_at(P, mx[j], my[j]) : 0u;
                 roff[j] = used ? bbase(P, ly[j] * Sh::kRingW + lx[j], 0, 0, kRP) : 0;
-                woff[j] = used ? bbase(P, (ly[j] + 1) * kWinW + lx[j] - 1 + Sh::kXOff, -(kWinW + 1), kWinW + 1, Sh::kWin) : 0;
+                // window cell: the image's own, or the mirror node's past a face that f does not wrap
+                const int cx = f_wraps(P.bc[0]) ? gx : mx[j], cy = f_wraps(P.bc[2]) ? gy : my[j];
+                woff[j] = used ? bbase(P, (cy - y0 + 2) * kWinW + cx - x0 + Sh::kXOff, -(kWinW + 1), kWinW + 1, Sh::kWin) : 0;
             }
             for (int p = z0 - 1; p <= z1; ++p, ++k) {
                 const int s = k % kStages;
@@ -1082,7 +1133,7 @@ k_fused_tma(const __grid_constant__ CUtensorMap map14, const __grid_constant__ C
                         continue;
                     }
                     float f[19], g[7];
-                    stage_pulls<Sh>(P, st + (j ? woff[1] : woff[0]), src, x, y, mz, f, g);
+                    stage_pulls<Sh, kFrozen>(P, st + (j ? woff[1] : woff[0]), src, x, y, mz, j ? at[1] : at[0], f, g);
                     const float rho = sum19(f), T = sum7(g);
                     const float psi2 = psi_squared(P, rho, T);
                     *out = make_float2(psi_of(psi2), rho);
@@ -1238,8 +1289,14 @@ cudaError_t launch_ghosts(const DevParams& P, int precision, void* pops, cudaStr
 }
 
 bool tma_eligible(const DevParams& P, int precision) {
-    return precision >= 0 && precision <= 2 && P.qt == 7 && P.nx >= 4 && P.ny >= 4 && f_wraps(P.bc[0]) && f_wraps(P.bc[1]) &&
-           f_wraps(P.bc[2]) && f_wraps(P.bc[3]) && !P.flow_off && !P.thermal_off && (!P.wet || precision == 0);
+    return precision >= 0 && precision <= 2 && P.qt == 7 && P.nx >= 4 && P.ny >= 4 && !P.flow_off &&
+           (!(P.wet || P.thermal_off) || precision == 0);
+}
+
+bool tma_runs(const DevParams& P, int precision, const StateBufs& B) {
+    // a frozen g is read in place (kFrozen); a frozen g that still is in streamed form (a checkpoint of
+    // a run with temperature) is left to the generic kernel
+    return tma_eligible(P, precision) && B.pull_f && (P.thermal_off ? !B.pull_g : B.pull_g != 0);
 }
 
 size_t tma_smem_bytes(int shape, int precision) {
@@ -1289,6 +1346,7 @@ int tma_tile_w(int shape) { return kTmaTX[shape]; }
 int tma_ghost_cols(int precision) { return precision == 0 ? 4 : 8; }   // 16 bytes of columns
 int tma_ghost_mode(const DevParams& P, int shape, int precision) {
     const int tx = tma_tile_w(shape), ty = kTmaTY[shape], gw = tma_ghost_cols(precision);
+    if (!f_wraps(P.bc[0]) && !f_wraps(P.bc[2])) return 3;   // no pull wraps: no ghost cells
     // TMA ghost boxes: ghost-column boxes (gw columns = 16 bytes) on 16-byte boundaries, at least
     // two tiles per axis (an edge tile is never both left and right, top and bottom), edge tiles at
     // least gw columns and 2 rows wide, and room for the gw ghost columns past nx in the padded rows
@@ -1303,18 +1361,18 @@ cudaError_t launch_fused(const DevParams& P, int precision, const StateBufs& B, 
     const int tiles_x = (P.nx + TX - 1) / TX, tiles_y = (P.ny + kTY - 1) / kTY;
     cudaError_t e = cudaSuccess;
     if (ghosts_written) *ghosts_written = false;
-    if (maps && maps->ok && B.pull_f && B.pull_g && tma_eligible(P, precision)) {
+    if (maps && maps->ok && tma_runs(P, precision, B)) {
         const int tx = kTmaTX[maps->shape], ty = kTmaTY[maps->shape];
         const int txs = (P.nx + tx - 1) / tx, tys = (P.ny + ty - 1) / ty;
         const int ctas = maps->sms < maps->items ? maps->sms : maps->items;
         if (ghosts_written) *ghosts_written = maps->ghosts != 0;
-#define GB300_TMA(TXV, TYV, ST, WET)                                                                           \
+#define GB300_TMA(TXV, TYV, ST, WET, FRO)                                                                      \
         {                                                                                                      \
             using SH = TmaShape<TXV, TYV, ST>;                                                                 \
-            e = cudaFuncSetAttribute(k_fused_tma<TXV, TYV, ST, WET>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+            e = cudaFuncSetAttribute(k_fused_tma<TXV, TYV, ST, WET, FRO>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                                      (int)SH::kSmem);                                                          \
             if (e != cudaSuccess) return e;                                                                    \
-            k_fused_tma<TXV, TYV, ST, WET><<<ctas, SH::kThreads, SH::kSmem, s>>>(                              \
+            k_fused_tma<TXV, TYV, ST, WET, FRO><<<ctas, SH::kThreads, SH::kSmem, s>>>(                              \
                 maps->m14[B.src_index], maps->m6[B.src_index], maps->mout[B.src_index ^ 1],                    \
                 maps->mout_top[B.src_index ^ 1], maps->mgcol[B.src_index ^ 1], maps->mgcol_top[B.src_index ^ 1], \
                 maps->mgrow[B.src_index ^ 1], maps->mgrow_right[B.src_index ^ 1], maps->mgcor[B.src_index ^ 1], \
@@ -1322,14 +1380,16 @@ cudaError_t launch_fused(const DevParams& P, int precision, const StateBufs& B, 
                 sums_next, B.phis,                                                                             \
                 B.flag, first, maps->zchunk, txs, tys, maps->items);                                           \
         }
-        // the wetting wall's solid plane is a separate instantiation (FP32 storage only), so that
-        // the kernel without it carries no trace of it
+        // the wetting wall's solid plane and a frozen temperature are separate instantiations (FP32 storage
+        // only), so that the kernel without them carries no trace of them
 #define GB300_TMA_CASE(I, X, Y)                                                                                \
         case I:                                                                                                \
-            if (precision == 0 && P.wet) GB300_TMA(X, Y, float, true)                                          \
-            else if (precision == 0) GB300_TMA(X, Y, float, false)                                             \
-            else if (precision == 1) GB300_TMA(X, Y, __nv_bfloat16, false)                                     \
-            else GB300_TMA(X, Y, __half, false)                                                                \
+            if (precision == 0 && P.thermal_off && P.wet) GB300_TMA(X, Y, float, true, true)                   \
+            else if (precision == 0 && P.thermal_off) GB300_TMA(X, Y, float, false, true)                      \
+            else if (precision == 0 && P.wet) GB300_TMA(X, Y, float, true, false)                              \
+            else if (precision == 0) GB300_TMA(X, Y, float, false, false)                                      \
+            else if (precision == 1) GB300_TMA(X, Y, __nv_bfloat16, false, false)                              \
+            else GB300_TMA(X, Y, __half, false, false)                                                         \
             break;
         switch (maps->shape) {
             GB300_TMA_SHAPES(GB300_TMA_CASE)

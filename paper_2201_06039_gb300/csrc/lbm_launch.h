@@ -54,7 +54,8 @@ struct TmaMaps {
     CUtensorMap mgcol[2], mgcol_top[2], mgrow[2], mgrow_right[2], mgcor[2];
     // ghost cells after a TMA step: 1 the edge tiles store them by TMA, 2 the edge nodes store their
     // periodic images directly (FP32 lattices whose nx is no multiple of the 16-byte band, or with
-    // one tile across an axis), 0 the refresh kernel writes them
+    // one tile across an axis), 0 the refresh kernel writes them, 3 none are read (f wraps on neither
+    // x nor y)
     int ghosts;
     bool ok;
     int sms;
@@ -80,6 +81,8 @@ bool fused_supported(const DevParams& P);
 // CTAs (partial sums) of one generic fused launch on P
 long long fused_blocks(const DevParams& P);
 bool tma_eligible(const DevParams& P, int precision);
+// does the TMA kernel take this step (given maps): eligible, and the state in the form it reads
+bool tma_runs(const DevParams& P, int precision, const StateBufs& B);
 // refresh the ghost columns / rows of a population buffer from their periodic images
 cudaError_t launch_ghosts(const DevParams& P, int precision, void* pops, cudaStream_t s);
 // tile shapes 0: 32 x 8, 1: 40 x 7, 2: 32 x 12, 3: 24 x 16 (window boxes tma_box_w x tma_box_h per
