@@ -555,7 +555,6 @@ int lbm_batch_init_fields(lbm_batch* b, const float* rho, const float* T, const 
         GB300_CK(cudaMemcpyAsync(stage + 2 * N, u, 3 * N * 4, cudaMemcpyHostToDevice, b->stream));
         du = stage + 2 * N;
     }
-    drop_batch_graphs(b);
     b->cur = 0;
     b->slot = 0;
     const size_t pb = pop_bytes(b->p.precision);

@@ -634,7 +634,7 @@ int lbm_init_fields(lbm_ctx* c, const float* rho, const float* T, const float* u
         CK(cudaMemcpyAsync(stage + 2 * N, u, 3 * N * 4, cudaMemcpyHostToDevice, c->stream));
         du = stage + 2 * N;
     }
-    drop_graphs(c);
+    // (captured step graphs stay: they hold the buffers, maps and parameters, which do not change here)
     c->cur = 0;
     c->slot = 0;
     CK(launch_init(c->dp, c->p.precision, c->pbuf(0), drho, dT, du, c->stream));
