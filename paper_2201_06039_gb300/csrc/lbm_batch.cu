@@ -711,6 +711,7 @@ int lbm_batch_get_totals(lbm_batch* b, double* sums) {
     if (!b->initialised) return fail(LBM_ESTATE, "lbm_batch_get_totals before lbm_batch_init_fields");
     for (int k = 0; k < b->n; ++k) {
         StateBufs B = b->bufs(k);
+        B.psirho = nullptr;   // sums only
         GB300_CK(launch_psi(b->dps[k], b->p.precision, B, b->sums(2) + 2 * k, b->stream));
     }
     GB300_CK(cudaMemcpyAsync(sums, b->sums(2), sizeof(double) * 2 * b->n, cudaMemcpyDeviceToHost, b->stream));

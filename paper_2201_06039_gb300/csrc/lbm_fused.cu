@@ -369,12 +369,16 @@ k_fused_batch(DevParams P, const BatchInst* __restrict__ insts, const BatchItem*
 // the ring holds the plane above; then u = (sum e f + F/2) / rho with F from the ring stencil.
 // Populations are read once (the ring's from L2) in place of twice by a psi pass and a moments pass.
 // kBatch: block b of the grid is item b of an ensemble's read-out table, its fields at field_off.
-template <typename S, int QT, bool kBatch>
+// kVel: the same pass as the first of a two-pass step with finite-difference div u: (psi, rho) and u of
+// every node (u as the collision forms it) and the FP64 sums of rho and T, in place of a psi pass and
+// a velocity pass that each read the populations.
+template <typename S, int QT, bool kBatch, bool kVel>
 __global__ void __launch_bounds__(FusedShape<kTY, QT>::kThreads, 2)
 k_readout(DevParams P0, const BatchInst* __restrict__ insts, const BatchItem* __restrict__ items,
           const S* __restrict__ src0, int pull_f, int pull_g, const double* __restrict__ sums_cur, int zchunk,
           float* __restrict__ orho, float* __restrict__ oux, float* __restrict__ ouy, float* __restrict__ ouz,
-          float* __restrict__ oT, int* flag) {
+          float* __restrict__ oT, int* flag, float2* __restrict__ psirho, float4* __restrict__ vel, double2* partial,
+          unsigned* counter, double* sums) {
     using Sh = FusedShape<kTY, QT>;
     __shared__ float2 ring[Sh::kRing * Sh::kRingPlane];
     int x0, y0, z0, z1, inst = 0;
@@ -433,6 +437,7 @@ k_readout(DevParams P0, const BatchInst* __restrict__ insts, const BatchItem* __
         o.jz = (f[5] - f[6]) + (f[11] - f[12]) - (f[13] - f[14]) + (f[15] - f[16]) - (f[17] - f[18]);
     };
     Node cur = {}, above = {};
+    float ra = 0.f, rc = 0.f, ta = 0.f, tc = 0.f;
     psi_pass(z0 - 1, above);
     psi_pass(z0, cur);
     for (int z = z0; z < z1; ++z) {
@@ -443,6 +448,18 @@ k_readout(DevParams P0, const BatchInst* __restrict__ insts, const BatchItem* __
                                                 ring + ((z + 1) % Sh::kRing) * Sh::kRingPlane,
                                                 bbase(P, slot, -(Sh::kRingW + 1), Sh::kRingW + 1, Sh::kRingPlane), Sh::kRingW);
             const float db = cur.rho - rho_ave;
+            if constexpr (kVel) {
+                const int d = (int)bidx(P, node_of(P, gx, gy, z), P.N);
+                const Forces F = total_force(P, cur.psi, rs.Fx, rs.Fy, rs.Fz, db);
+                const float inv_rho = __fdividef(1.f, cur.rho);
+                psirho[d] = make_float2(cur.psi, cur.rho);
+                vel[d] = make_float4((cur.jx + 0.5f * F.Fx) * inv_rho, (cur.jy + 0.5f * F.Fy) * inv_rho,
+                                     (cur.jz + 0.5f * F.Fz) * inv_rho, 0.f);
+                kahan_add(ra, rc, cur.rho);
+                kahan_add(ta, tc, cur.T);
+                cur = above;
+                continue;
+            }
             const float Fx = __fmaf_rn(cur.psi, rs.Fx, __fmul_rn(db, P.gx)), Fy = __fmaf_rn(cur.psi, rs.Fy, __fmul_rn(db, P.gy)),
                         Fz = __fmaf_rn(cur.psi, rs.Fz, __fmul_rn(db, P.gz));
             const float inv = 1.f / cur.rho;
@@ -457,6 +474,15 @@ k_readout(DevParams P0, const BatchInst* __restrict__ insts, const BatchItem* __
         cur = above;
     }
     if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(flag, 1);
+    if constexpr (kVel) {
+        __shared__ double red_a[Sh::kThreads / 32], red_b[Sh::kThreads / 32];
+        __shared__ int is_last;
+        const int bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
+        block_partial<Sh::kThreads>((double)ra - (double)rc, (double)ta - (double)tc, partial, bid, threadIdx.x, 0, red_a,
+                                    red_b);
+        finish_sums<Sh::kThreads>(partial, gridDim.x * gridDim.y * gridDim.z, counter, sums, threadIdx.x, 0, red_a, red_b,
+                                  &is_last);
+    }
 }
 
 // ================================================================ TMA producer / consumer kernel
@@ -1428,12 +1454,17 @@ cudaError_t launch_fused(const DevParams& P, int precision, const StateBufs& B, 
     return cudaGetLastError();
 }
 
-// planes of a read-out block: about six blocks for each of the two resident on an SM, so that the
-// last wave is short, at least two planes (a block reads two more than it writes)
+// Planes of a read-out block (it reads two more than it writes): twelve blocks an SM where that leaves
+// at least five planes (128^3: 5 planes 195 us, 8 planes 223), else the fewest planes, up to six, whose
+// blocks make one round of two an SM (64 x 64 x 96: 6 planes in place of 2, 46 -> 39 us a call).
 static int zchunk_readout(const DevParams& P, long long tiles) {
-    const long long target = (long long)device_sms() * 12;
-    const int chunks = (int)std::max<long long>(1, std::min<long long>(target / tiles, P.nz / 2));
-    return (P.nz + chunks - 1) / chunks;
+    const long long sms = device_sms();
+    const int chunks = (int)std::max<long long>(1, std::min<long long>(12 * sms / tiles, P.nz));
+    int zc = (P.nz + chunks - 1) / chunks;
+    if (zc >= 5) return zc;
+    for (zc = 1; zc < 6; ++zc)
+        if (tiles * ((P.nz + zc - 1) / zc) <= 2 * sms) return zc;
+    return zc;
 }
 
 cudaError_t launch_readout(const DevParams& P, int precision, const StateBufs& B, const double* sums_cur, float* rho,
@@ -1442,8 +1473,9 @@ cudaError_t launch_readout(const DevParams& P, int precision, const StateBufs& B
     const int zc = zchunk_readout(P, (long long)tiles_x * tiles_y);
     const dim3 grid(tiles_x, tiles_y, (P.nz + zc - 1) / zc);
 #define GB300_READ(S, QT)                                                                                      \
-    k_readout<S, QT, false><<<grid, FusedShape<kTY, QT>::kThreads, 0, s>>>(P, nullptr, nullptr, (const S*)B.src, \
-                                                                           B.pull_f, B.pull_g, sums_cur, zc, rho, ux, uy, uz, T, B.flag)
+    k_readout<S, QT, false, false><<<grid, FusedShape<kTY, QT>::kThreads, 0, s>>>(                             \
+        P, nullptr, nullptr, (const S*)B.src, B.pull_f, B.pull_g, sums_cur, zc, rho, ux, uy, uz, T, B.flag,    \
+        nullptr, nullptr, nullptr, nullptr, nullptr)
     if (P.qt == 19) {
         if (precision != 0) return cudaErrorInvalidValue;
         GB300_READ(float, 19);
@@ -1459,12 +1491,37 @@ cudaError_t launch_readout(const DevParams& P, int precision, const StateBufs& B
     return cudaGetLastError();
 }
 
+cudaError_t launch_psi_velocity(const DevParams& P, int precision, const StateBufs& B, const double* sums_cur,
+                                double* sums, cudaStream_t s) {
+    const int tiles_x = (P.nx + TX - 1) / TX, tiles_y = (P.ny + kTY - 1) / kTY;
+    const int zc = zchunk_readout(P, (long long)tiles_x * tiles_y);
+    const dim3 grid(tiles_x, tiles_y, (P.nz + zc - 1) / zc);
+#define GB300_VEL(S, QT)                                                                                       \
+    k_readout<S, QT, false, true><<<grid, FusedShape<kTY, QT>::kThreads, 0, s>>>(                              \
+        P, nullptr, nullptr, (const S*)B.src, B.pull_f, B.pull_g, sums_cur, zc, nullptr, nullptr, nullptr, nullptr, \
+        nullptr, B.flag, B.psirho, B.vel, B.partial, B.counter, sums)
+    if (P.qt == 19) {
+        if (precision != 0) return cudaErrorInvalidValue;
+        GB300_VEL(float, 19);
+    } else {
+        switch (precision) {
+        case 0: GB300_VEL(float, 7); break;
+        case 1: GB300_VEL(__nv_bfloat16, 7); break;
+        case 2: GB300_VEL(__half, 7); break;
+        default: return cudaErrorInvalidValue;
+        }
+    }
+#undef GB300_VEL
+    return cudaGetLastError();
+}
+
 cudaError_t launch_readout_batch(const DevParams& P, int precision, const BatchInst* insts, const BatchItem* items,
                                  int n_items, const StateBufs& B, const double* sums_cur, float* rho, float* ux,
                                  float* uy, float* uz, float* T, cudaStream_t s) {
 #define GB300_READ(S)                                                                                          \
-    k_readout<S, 7, true><<<n_items, FusedShape<kTY>::kThreads, 0, s>>>(P, insts, items, (const S*)B.src, B.pull_f, \
-                                                                        B.pull_g, sums_cur, 0, rho, ux, uy, uz, T, B.flag)
+    k_readout<S, 7, true, false><<<n_items, FusedShape<kTY>::kThreads, 0, s>>>(                                \
+        P, insts, items, (const S*)B.src, B.pull_f, B.pull_g, sums_cur, 0, rho, ux, uy, uz, T, B.flag, nullptr, \
+        nullptr, nullptr, nullptr, nullptr)
     switch (precision) {
     case 0: GB300_READ(float); break;
     case 1: GB300_READ(__nv_bfloat16); break;

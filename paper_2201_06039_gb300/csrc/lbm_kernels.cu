@@ -1,5 +1,7 @@
 // Two-pass kernels of the lattice update, initialisation, moments and deterministic
 // FP64 reductions.  See lbm_device.cuh for the per-node arithmetic.
+#include <algorithm>
+
 #include "lbm_launch.h"
 
 namespace gb300lbm {
@@ -75,24 +77,31 @@ __global__ void __launch_bounds__(TPB) k_init(DevParams P, S* __restrict__ pops,
 }
 
 // ---------------------------------------------------------------- psi / EOS pass (S1-S2)
+// (psi, rho) of every node (psirho; NULL: sums only) and the FP64 sums of rho and T.  A block takes
+// zchunk planes of its 32 x 8 columns, so that a thread adds its nodes in FP64 and the block reduces
+// once: with a reduction per plane (10 FP64 shuffle-adds a warp and node, at the FP64 rate) the pass
+// took 32 us on 64 x 64 x 96, three times its reads.
 template <typename S, int QT>
 __global__ void __launch_bounds__(TPB) k_psi(DevParams P, const S* __restrict__ fs, int pull_f, int pull_g, float2* __restrict__ psirho,
-                                            double2* partial, unsigned* counter, double* sums, int* flag) {
-    int x = blockIdx.x * TPB_X + threadIdx.x, y = blockIdx.y * TPB_Y + threadIdx.y, z = blockIdx.z;
+                                            double2* partial, unsigned* counter, double* sums, int* flag, int zchunk) {
+    int x = blockIdx.x * TPB_X + threadIdx.x, y = blockIdx.y * TPB_Y + threadIdx.y;
+    const int z1 = min(P.nz, (int)(blockIdx.z + 1) * zchunk);
     double ra = 0.0, ta = 0.0;
     int bad = 0;
     if (x < P.nx && y < P.ny) {
-        int i = sidx(P, x, y, z);
-        Nbr n = make_nbr(P, x, y, z);
-        float f[19], g[QT];
-        load_f<S>(P, fs, pull_f, i, x, y, z, n, f);
-        Therm<QT>::template load<S>(P, fs, pull_g, i, x, y, z, n, g);
-        float rho = sum19(f), T = Therm<QT>::sum(g);
-        float psi2 = psi_squared(P, rho, T);
-        bad = !(psi2 > 0.f) || !isfinite(rho) || !isfinite(T);
-        psirho[bidx(P, node_of(P, x, y, z), P.N)] = make_float2(psi_of(psi2), rho);
-        ra = rho;
-        ta = T;
+        for (int z = blockIdx.z * zchunk; z < z1; ++z) {
+            int i = sidx(P, x, y, z);
+            Nbr n = make_nbr(P, x, y, z);
+            float f[19], g[QT];
+            load_f<S>(P, fs, pull_f, i, x, y, z, n, f);
+            Therm<QT>::template load<S>(P, fs, pull_g, i, x, y, z, n, g);
+            float rho = sum19(f), T = Therm<QT>::sum(g);
+            float psi2 = psi_squared(P, rho, T);
+            bad |= !(psi2 > 0.f) || !isfinite(rho) || !isfinite(T);
+            if (psirho) psirho[bidx(P, node_of(P, x, y, z), P.N)] = make_float2(psi_of(psi2), rho);
+            ra += rho;
+            ta += T;
+        }
     }
     if (__syncthreads_or(bad) && threadIdx.x == 0 && threadIdx.y == 0) atomicOr(flag, 1);
     if (sums) grid_sum2<TPB>(ra, ta, partial, counter, sums);
@@ -137,30 +146,6 @@ __device__ __forceinline__ Stencil stencil(const DevParams& P, const float2* __r
     return s;
 }
 
-// ---------------------------------------------------------------- velocity pass
-// u = (sum e f + F/2) / rho (Eq. 10, total force F) of every node, for the finite-difference
-// div u of the collide pass (divu_mode 1); same arithmetic as the collision's u.
-template <typename S>
-__global__ void __launch_bounds__(TPB) k_velocity(DevParams P, const S* __restrict__ fs, int pull_f,
-                                                 const float2* __restrict__ psirho,
-                                                 const double* __restrict__ sums_cur, float4* __restrict__ vel) {
-    int x = blockIdx.x * TPB_X + threadIdx.x, y = blockIdx.y * TPB_Y + threadIdx.y, z = blockIdx.z;
-    if (x >= P.nx || y >= P.ny) return;
-    int i = sidx(P, x, y, z), d = (int)bidx(P, node_of(P, x, y, z), P.N);
-    Nbr n = make_nbr(P, x, y, z);
-    float f[19];
-    load_f<S>(P, fs, pull_f, i, x, y, z, n, f);
-    float rho = sum19(f);
-    float jx = (f[1] - f[2]) + (f[7] - f[8]) + (f[9] - f[10]) + (f[11] - f[12]) + (f[13] - f[14]);
-    float jy = (f[3] - f[4]) + (f[7] - f[8]) - (f[9] - f[10]) + (f[15] - f[16]) + (f[17] - f[18]);
-    float jz = (f[5] - f[6]) + (f[11] - f[12]) - (f[13] - f[14]) + (f[15] - f[16]) - (f[17] - f[18]);
-    float2 me = __ldg(psirho + d);
-    Stencil st = stencil(P, psirho, x, y, z, n);
-    const Forces F = total_force(P, me.x, st.x.x, st.y.x, st.z.x, rho - buoyancy_ref(P, sums_cur[0], P.inv_N));
-    const float inv_rho = __fdividef(1.f, rho);
-    vel[d] = make_float4((jx + 0.5f * F.Fx) * inv_rho, (jy + 0.5f * F.Fy) * inv_rho, (jz + 0.5f * F.Fz) * inv_rho, 0.f);
-}
-
 // Does the gradient stencil of (x, y, z) reach past a wall or outflow face?  There div u stays
 // Eq. 48 in divu_mode 1.
 __device__ __forceinline__ bool next_to_solid(const DevParams& P, int x, int y, int z) {
@@ -197,7 +182,7 @@ __device__ __forceinline__ float fd_divergence(const DevParams& P, const float4*
 
 // ---------------------------------------------------------------- stream-collide pass (S3-S12)
 template <typename S, int QT>
-__global__ void __launch_bounds__(TPB) k_collide(DevParams P, const S* __restrict__ fs, S* __restrict__ fd,
+__global__ void __launch_bounds__(TPB, QT == 7 ? 3 : 2) k_collide(DevParams P, const S* __restrict__ fs, S* __restrict__ fd,
                                                 int pull_f, int pull_g,
                                                 const float2* __restrict__ psirho, const double* __restrict__ sums_cur,
                                                 float* __restrict__ phis, int first, const float4* __restrict__ vel) {
@@ -276,9 +261,12 @@ cudaError_t launch_init(const DevParams& P, int precision, void* pops, const flo
 }
 
 cudaError_t launch_psi(const DevParams& P, int precision, const StateBufs& B, double* sums, cudaStream_t s) {
-    dim3 blk(TPB_X, TPB_Y);
-    GB300_DISPATCH_QT(P, precision, (k_psi<S, QT><<<grid_of(P), blk, 0, s>>>(P, (const S*)B.src, B.pull_f, B.pull_g, B.psirho,
-                                                                    B.partial, B.counter, sums, B.flag)));
+    dim3 blk(TPB_X, TPB_Y), grid = grid_of(P);
+    // one round of three blocks an SM, at most 16 planes a block
+    const int zc = (int)std::max(1LL, std::min(16LL, ((long long)grid.x * grid.y * grid.z + 455) / 456));
+    grid.z = (P.nz + zc - 1) / zc;
+    GB300_DISPATCH_QT(P, precision, (k_psi<S, QT><<<grid, blk, 0, s>>>(P, (const S*)B.src, B.pull_f, B.pull_g, B.psirho,
+                                                                       B.partial, B.counter, sums, B.flag, zc)));
     return cudaGetLastError();
 }
 
@@ -355,14 +343,6 @@ cudaError_t launch_wall_table(const DevParams& P, int precision, const void* fs,
                               cudaStream_t s) {
     const dim3 grid((P.nx + 127) / 128, P.ny);
     GB300_DISPATCH(precision, (k_wall_table<S><<<grid, 128, 0, s>>>(P, (const S*)fs, pull_f, tab)));
-    return cudaGetLastError();
-}
-
-cudaError_t launch_velocity(const DevParams& P, int precision, const StateBufs& B, const double* sums_cur,
-                            cudaStream_t s) {
-    dim3 blk(TPB_X, TPB_Y);
-    GB300_DISPATCH(precision, (k_velocity<S><<<grid_of(P), blk, 0, s>>>(P, (const S*)B.src, B.pull_f, B.psirho,
-                                                                         sums_cur, B.vel)));
     return cudaGetLastError();
 }
 

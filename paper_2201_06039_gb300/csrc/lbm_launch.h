@@ -26,19 +26,20 @@ int reduce_blocks_psi(const DevParams& P);
 cudaError_t launch_init(const DevParams& P, int precision, void* pops, const float* rho, const float* T,
                         const float* u, cudaStream_t s);
 
-// psi/EOS pass: rho, T, psi of every node; optional FP64 sums (rho, T) into sums[0..1].
+// psi/EOS pass: (psi, rho) of every node into B.psirho (nullable); optional FP64 sums (rho, T) into
+// sums[0..1].
 cudaError_t launch_psi(const DevParams& P, int precision, const StateBufs& B, double* sums,
                        cudaStream_t s);
 
-// stream-collide pass of the two-pass variant.
-// u = (sum e f + F/2) / rho of every node into B.vel (finite-difference div u)
+// the psi pass with u = (sum e f + F/2) / rho of every node into B.vel (finite-difference div u)
+cudaError_t launch_psi_velocity(const DevParams& P, int precision, const StateBufs& B, const double* sums_cur,
+                                double* sums, cudaStream_t s);
 cudaError_t launch_wall_params(const DevParams& P, float2* par, cudaStream_t s);
 cudaError_t launch_wall_map(const DevParams& P, const float* phi, const float* drho, float2* par, int* bad,
                             int write, cudaStream_t s);
 cudaError_t launch_wall_table(const DevParams& P, int precision, const void* fs, int pull_f, float2* tab,
                               cudaStream_t s);
-cudaError_t launch_velocity(const DevParams& P, int precision, const StateBufs& B, const double* sums_cur,
-                            cudaStream_t s);
+// stream-collide pass of the two-pass variant.
 cudaError_t launch_collide(const DevParams& P, int precision, const StateBufs& B,
                            const double* sums_cur, int first, cudaStream_t s);
 
