@@ -95,6 +95,7 @@ struct lbm_ctx {
     long long steps;
     int variant;   // LBM_KERNEL_TWO_PASS or LBM_KERNEL_FUSED
     TmaMaps maps;
+    TmaMaps read_maps;             // of the read-out's tile shape
     int plan_shape, plan_zchunk;   // TMA plan pinned by lbm_select_plan (-1 / 0: automatic)
     GraphEntry graphs[kGraphCache];
     int n_graphs;
@@ -591,7 +592,8 @@ int lbm_create(const lbm_params* p, lbm_ctx** out) {
     c->plan_shape = -1;
     c->plan_zchunk = 0;
     c->dp.check_flag = (int*)(c->base + c->L.flag);
-    if (c->variant == LBM_KERNEL_FUSED && p->use_tma != 0) make_tma_maps(c);
+    if (c->variant == LBM_KERNEL_FUSED && p->use_tma != 0 && make_tma_maps(c))
+        build_tma_maps(c->dp, c->p.precision, c->pbuf(0), c->pbuf(1), 0, tma_read_shape(), 0, max_partials(c->dp), &c->read_maps);
     cudaError_t e = cudaMemsetAsync(c->base + c->L.sums, 0, c->L.flag + sizeof(int) - c->L.sums, c->stream);
     if (e == cudaSuccess && c->dp.wet) {   // scheme 0: the table is constant; scheme 1: refreshed every step
         c->dp.wall_tab = (const float2*)(c->base + c->L.wall);
@@ -701,7 +703,8 @@ int lbm_get_moments(lbm_ctx* c, float* rho, float* ux, float* uy, float* uz, flo
     float* outs[5] = {rho, ux, uy, uz, T};
     float* dst[5];
     for (int k = 0; k < 5; ++k) dst[k] = outs[k] ? (is_device_ptr(outs[k]) ? outs[k] : stage + k * N) : nullptr;
-    CK(launch_readout(c->dp, c->p.precision, B, c->sums(c->slot), dst[0], dst[1], dst[2], dst[3], dst[4], c->stream));
+    CK(launch_readout(c->dp, c->p.precision, B, c->sums(c->slot), dst[0], dst[1], dst[2], dst[3], dst[4], c->stream,
+                      c->maps.ok ? &c->read_maps : nullptr));
     for (int k = 0; k < 5; ++k)
         if (outs[k] && dst[k] != outs[k])
             CK(cudaMemcpyAsync(outs[k], dst[k], N * 4, cudaMemcpyDeviceToHost, c->stream));

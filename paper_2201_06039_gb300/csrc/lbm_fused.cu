@@ -363,6 +363,24 @@ k_fused_batch(DevParams P, const BatchInst* __restrict__ insts, const BatchItem*
 }
 
 // ================================================================ read-out
+struct ReadFields {   // device arrays, each nullable
+    float *rho, *ux, *uy, *uz, *T;
+};
+// the fields of one node: u = (j + F/2) / rho, F = F_m + (rho - rho_ave) g
+__device__ __forceinline__ void write_fields(const DevParams& P, const ReadFields& out, long long d, float rho, float T,
+                                             float psi, float jx, float jy, float jz, const RingStencil& rs, float rho_ave) {
+    const float db = rho - rho_ave;
+    const float Fx = __fmaf_rn(psi, rs.Fx, __fmul_rn(db, P.gx)), Fy = __fmaf_rn(psi, rs.Fy, __fmul_rn(db, P.gy)),
+                Fz = __fmaf_rn(psi, rs.Fz, __fmul_rn(db, P.gz));
+    const float inv = 1.f / rho;
+    const bool fz = P.flow_off != 0;
+    if (out.rho) out.rho[d] = rho;
+    if (out.ux) out.ux[d] = fz ? 0.f : (jx + 0.5f * Fx) * inv;
+    if (out.uy) out.uy[d] = fz ? 0.f : (jy + 0.5f * Fy) * inv;
+    if (out.uz) out.uz[d] = fz ? 0.f : (jz + 0.5f * Fz) * inv;
+    if (out.T) out.T[d] = T;
+}
+
 // Macroscopic fields in one pass over the populations: a block marches a 32 x 8 tile through a chunk
 // of planes; every thread pulls its node (or a node of the ring around the tile), puts (psi, rho) into
 // a four-plane shared ring and keeps rho, T and the first moment of its node for one plane, until
@@ -376,8 +394,7 @@ template <typename S, int QT, bool kBatch, bool kVel>
 __global__ void __launch_bounds__(FusedShape<kTY, QT>::kThreads, 2)
 k_readout(DevParams P0, const BatchInst* __restrict__ insts, const BatchItem* __restrict__ items,
           const S* __restrict__ src0, int pull_f, int pull_g, const double* __restrict__ sums_cur, int zchunk,
-          float* __restrict__ orho, float* __restrict__ oux, float* __restrict__ ouy, float* __restrict__ ouz,
-          float* __restrict__ oT, int* flag, float2* __restrict__ psirho, float4* __restrict__ vel, double2* partial,
+          ReadFields out, int* flag, float2* __restrict__ psirho, float4* __restrict__ vel, double2* partial,
           unsigned* counter, double* sums) {
     using Sh = FusedShape<kTY, QT>;
     __shared__ float2 ring[Sh::kRing * Sh::kRingPlane];
@@ -447,8 +464,8 @@ k_readout(DevParams P0, const BatchInst* __restrict__ insts, const BatchItem* __
             const RingStencil rs = ring_stencil(ring + ((z + 3) % Sh::kRing) * Sh::kRingPlane, ring + (z % Sh::kRing) * Sh::kRingPlane,
                                                 ring + ((z + 1) % Sh::kRing) * Sh::kRingPlane,
                                                 bbase(P, slot, -(Sh::kRingW + 1), Sh::kRingW + 1, Sh::kRingPlane), Sh::kRingW);
-            const float db = cur.rho - rho_ave;
             if constexpr (kVel) {
+                const float db = cur.rho - rho_ave;
                 const int d = (int)bidx(P, node_of(P, gx, gy, z), P.N);
                 const Forces F = total_force(P, cur.psi, rs.Fx, rs.Fy, rs.Fz, db);
                 const float inv_rho = __fdividef(1.f, cur.rho);
@@ -460,16 +477,8 @@ k_readout(DevParams P0, const BatchInst* __restrict__ insts, const BatchItem* __
                 cur = above;
                 continue;
             }
-            const float Fx = __fmaf_rn(cur.psi, rs.Fx, __fmul_rn(db, P.gx)), Fy = __fmaf_rn(cur.psi, rs.Fy, __fmul_rn(db, P.gy)),
-                        Fz = __fmaf_rn(cur.psi, rs.Fz, __fmul_rn(db, P.gz));
-            const float inv = 1.f / cur.rho;
-            const bool fz = P.flow_off != 0;
-            const long long d = field_off + bidx(P, node_of(P, gx, gy, z), P.N);
-            if (orho) orho[d] = cur.rho;
-            if (oux) oux[d] = fz ? 0.f : (cur.jx + 0.5f * Fx) * inv;
-            if (ouy) ouy[d] = fz ? 0.f : (cur.jy + 0.5f * Fy) * inv;
-            if (ouz) ouz[d] = fz ? 0.f : (cur.jz + 0.5f * Fz) * inv;
-            if (oT) oT[d] = cur.T;
+            write_fields(P, out, field_off + bidx(P, node_of(P, gx, gy, z), P.N), cur.rho, cur.T, cur.psi, cur.jx, cur.jy,
+                         cur.jz, rs, rho_ave);
         }
         cur = above;
     }
@@ -816,7 +825,7 @@ __device__ __forceinline__ void nb_arrive(int id, int nthreads) {
 // halo); the copy warp's next arrival on RING(s) follows its OUT_FULL(s) sync of the previous use of
 // s, whose arrivals follow that use's RING(s); and the compute warps' next arrival on OUT_FULL(s)
 // follows their RING(s) sync of the next use of s, which needs that arrival of the copy warp.
-template <int TX_, int TY_, typename S, bool kWet, bool kFrozen>
+template <int TX_, int TY_, typename S, bool kWet, bool kFrozen, bool kRead>
 __global__ void __maxnreg__((TmaShape<TX_, TY_, S>::kMaxRegs))
 k_fused_tma(const __grid_constant__ CUtensorMap map14, const __grid_constant__ CUtensorMap map6,
             const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_out_top,
@@ -825,7 +834,8 @@ k_fused_tma(const __grid_constant__ CUtensorMap map14, const __grid_constant__ C
             const __grid_constant__ CUtensorMap map_gcor, int ghosts, DevParams P, const S* __restrict__ src,
             S* __restrict__ dst,
             const double* __restrict__ sums_cur, double2* partial, unsigned* counter, double* sums_next,
-            float* __restrict__ phis, int* flag, int first, int zchunk, int tiles_x, int tiles_y, int n_items) {
+            float* __restrict__ phis, int* flag, int first, int zchunk, int tiles_x, int tiles_y, int n_items,
+            ReadFields out) {
     using Sh = TmaShape<TX_, TY_, S>;
     constexpr int kWinW = Sh::kWinW, kStages = Sh::kStages, kRing = Sh::kRing, kRP = Sh::kRingPlane;
     constexpr int kComp = Sh::kCompThreads, kGW = Sh::kGW;
@@ -885,7 +895,7 @@ k_fused_tma(const __grid_constant__ CUtensorMap map14, const __grid_constant__ C
         auto load = [&]() {
             const int s = kl % kStages;
             if (lane == 0) {
-                if (P.test_stall && kl == 0) {
+                if (!kRead && P.test_stall && kl == 0) {
                     // timeout-path test: the first stage's data never comes; the copy warp waits
                     // (bounded) on a barrier nothing completes, then releases the stage empty
                     if (!mbar_wait(&stall_bar, 0u)) {
@@ -922,7 +932,7 @@ k_fused_tma(const __grid_constant__ CUtensorMap map14, const __grid_constant__ C
             // nodes itself (a tensor store clipped at nx inside a 16-byte unit also writes the
             // ghost columns past nx, which the first tile column's nodes write)
             const bool direct_tile = ghosts == 2 && st.x0 + TX_ > P.nx && P.nx % kGW != 0;
-            if (st.p > st.z0 && lane == 0 && !abort_flag && !direct_tile) {   // the stage holds collided plane p - 1
+            if (!kRead && st.p > st.z0 && lane == 0 && !abort_flag && !direct_tile) {   // the stage holds collided plane p - 1
                 const int z = st.p - 1, x0 = st.x0, y0 = st.y0;
                 // box (x, slot, y, z) at the tile origin (x a multiple of 4 floats); the last tile
                 // row uses the map whose box holds exactly its rows, so a box never reaches past
@@ -1005,7 +1015,7 @@ k_fused_tma(const __grid_constant__ CUtensorMap map14, const __grid_constant__ C
             const int rw = min(TX_, P.nx - x0);
             float r_sum = 0.f, r_c = 0.f, t_sum = 0.f, t_c = 0.f;
             // phi_s history of the thread's node, loaded one plane ahead of its use
-            float ph_next = owner ? phis[bidx(P, node_of(P, gx, gy, z0), P.N)] : 0.f;
+            float ph_next = !kRead && owner ? phis[bidx(P, node_of(P, gx, gy, z0), P.N)] : 0.f;
 
             // pull plane p (stage use k) into (fo, go), put the node's (psi, rho) into ring plane k
             auto pull_plane = [&](int p, float* fo, float* go, float& ro, float& To, float& po) {
@@ -1090,6 +1100,38 @@ k_fused_tma(const __grid_constant__ CUtensorMap map14, const __grid_constant__ C
                 if (owner) phis[bidx(P, node_of(P, gx, gy, z), P.N)] = ph;
             };
 
+            if constexpr (kRead) {
+                // read-out: of a plane's populations only rho, T and the first moment are kept until
+                // the ring holds the plane above
+                float f[19], g[7], rho = 0.f, T = 0.f, psi = 0.f, jx = 0.f, jy = 0.f, jz = 0.f;
+                float rho_n = 0.f, T_n = 0.f, psi_n = 0.f;
+                auto pull = [&](int p, float& r, float& t, float& ps) {
+                    pull_plane(p, f, g, r, t, ps);
+                    nb_arrive(bar_out_full((k - 1) % kStages), Sh::kCntOut);   // nothing to store
+                };
+                auto moment = [&] {
+                    jx = (f[1] - f[2]) + (f[7] - f[8]) + (f[9] - f[10]) + (f[11] - f[12]) + (f[13] - f[14]);
+                    jy = (f[3] - f[4]) + (f[7] - f[8]) - (f[9] - f[10]) + (f[15] - f[16]) + (f[17] - f[18]);
+                    jz = (f[5] - f[6]) + (f[11] - f[12]) - (f[13] - f[14]) + (f[15] - f[16]) - (f[17] - f[18]);
+                };
+                pull(z0 - 1, rho_n, T_n, psi_n);
+                pull(z0, rho, T, psi);
+                moment();
+#pragma unroll 1
+                for (int z = z0; z < z1; ++z) {
+                    pull(z + 1, rho_n, T_n, psi_n);
+                    if (owner) {
+                        const RingStencil rs = ring_stencil(ring + ((k - 3) % kRing) * kRP, ring + ((k - 2) % kRing) * kRP,
+                                                            ring + ((k - 1) % kRing) * kRP, slot, Sh::kRingW);
+                        write_fields(P, out, bidx(P, node_of(P, gx, gy, z), P.N), rho, T, psi, jx, jy, jz, rs, rho_ave);
+                    }
+                    moment();
+                    rho = rho_n;
+                    T = T_n;
+                    psi = psi_n;
+                }
+                continue;
+            }
             // the populations of the plane being collided (a) and of the plane pulled ahead (b)
             float fa[19], ga[7], ra = 0.f, Ta = 0.f, pa = 0.f;
             float fb[19], gb[7], rb = 0.f, Tb = 0.f, pb = 0.f;
@@ -1114,7 +1156,7 @@ k_fused_tma(const __grid_constant__ CUtensorMap map14, const __grid_constant__ C
                                  kBarComp, red_a, red_b);
         }
         if (bad) atomicOr(flag, 1);
-        finish_sums<kComp>(partial, n_items, counter, sums_next, ct, kBarComp, red_a, red_b, &is_last);
+        if constexpr (!kRead) finish_sums<kComp>(partial, n_items, counter, sums_next, ct, kBarComp, red_a, red_b, &is_last);
     } else {
         // ------------------------------------------------------------ halo psi (two warps)
         const int h = tid - 32 * (Sh::kLeadWarps + Sh::kCompWarps);
@@ -1237,6 +1279,9 @@ constexpr int kTmaTX[kNumTmaShapes] = {32, 40, 32, 24, 40, 40};
 constexpr int kTmaTY[kNumTmaShapes] = {8, 7, 12, 16, 8, 10};
 constexpr double kTmaRate[kNumTmaShapes] = {1.0, 0.97, 1.17, 1.06, 1.08, 1.11};
 
+// tile shape of the read-out's instantiation of the kernel
+constexpr int kReadShape = 2;
+
 // Modelled time of a plan: items (tile, z-chunk) go round robin to the persistent CTAs; a plane of an
 // item costs its tile nodes over the shape's rate, and an item two planes more (its psi-only planes).
 // The busiest CTA counts.  The model holds down to chunks of one plane: a 32^3 lattice measured
@@ -1339,6 +1384,7 @@ void tma_plan_for(const DevParams& P, int ctas, int forced_shape, int forced_zch
 }
 
 int tma_num_shapes() { return kNumTmaShapes; }
+int tma_read_shape() { return kReadShape; }
 double tma_rate(int shape) { return kTmaRate[shape]; }
 
 int tma_zchunk_candidates(const DevParams& P, int ctas, int shape, int* zcs, int max) {
@@ -1381,6 +1427,22 @@ int tma_ghost_mode(const DevParams& P, int shape, int precision) {
 }
 int tma_tile_h(int shape) { return kTmaTY[shape]; }
 
+// one launch of the TMA kernel on the enclosing function's P, B, maps, ctas, txs, tys, first, fields
+#define GB300_TMA(TXV, TYV, ST, WET, FRO, READ)                                                                \
+        {                                                                                                      \
+            using SH = TmaShape<TXV, TYV, ST>;                                                                 \
+            e = cudaFuncSetAttribute(k_fused_tma<TXV, TYV, ST, WET, FRO, READ>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                                     (int)SH::kSmem);                                                          \
+            if (e != cudaSuccess) return e;                                                                    \
+            k_fused_tma<TXV, TYV, ST, WET, FRO, READ><<<ctas, SH::kThreads, SH::kSmem, s>>>(                              \
+                maps->m14[B.src_index], maps->m6[B.src_index], maps->mout[B.src_index ^ 1],                    \
+                maps->mout_top[B.src_index ^ 1], maps->mgcol[B.src_index ^ 1], maps->mgcol_top[B.src_index ^ 1], \
+                maps->mgrow[B.src_index ^ 1], maps->mgrow_right[B.src_index ^ 1], maps->mgcor[B.src_index ^ 1], \
+                maps->ghosts, P, (const ST*)B.src, (ST*)B.dst, sums_cur, B.partial, B.counter,                  \
+                sums_next, B.phis,                                                                             \
+                B.flag, first, maps->zchunk, txs, tys, maps->items, fields);                                   \
+        }
+
 cudaError_t launch_fused(const DevParams& P, int precision, const StateBufs& B, const double* sums_cur,
                          double* sums_next, int first, cudaStream_t s, const TmaMaps* maps, bool* ghosts_written) {
     using Sh = FusedShape<kTY>;
@@ -1392,37 +1454,23 @@ cudaError_t launch_fused(const DevParams& P, int precision, const StateBufs& B, 
         const int txs = (P.nx + tx - 1) / tx, tys = (P.ny + ty - 1) / ty;
         const int ctas = maps->sms < maps->items ? maps->sms : maps->items;
         if (ghosts_written) *ghosts_written = maps->ghosts != 0;
-#define GB300_TMA(TXV, TYV, ST, WET, FRO)                                                                      \
-        {                                                                                                      \
-            using SH = TmaShape<TXV, TYV, ST>;                                                                 \
-            e = cudaFuncSetAttribute(k_fused_tma<TXV, TYV, ST, WET, FRO>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                     (int)SH::kSmem);                                                          \
-            if (e != cudaSuccess) return e;                                                                    \
-            k_fused_tma<TXV, TYV, ST, WET, FRO><<<ctas, SH::kThreads, SH::kSmem, s>>>(                              \
-                maps->m14[B.src_index], maps->m6[B.src_index], maps->mout[B.src_index ^ 1],                    \
-                maps->mout_top[B.src_index ^ 1], maps->mgcol[B.src_index ^ 1], maps->mgcol_top[B.src_index ^ 1], \
-                maps->mgrow[B.src_index ^ 1], maps->mgrow_right[B.src_index ^ 1], maps->mgcor[B.src_index ^ 1], \
-                maps->ghosts, P, (const ST*)B.src, (ST*)B.dst, sums_cur, B.partial, B.counter,                  \
-                sums_next, B.phis,                                                                             \
-                B.flag, first, maps->zchunk, txs, tys, maps->items);                                           \
-        }
+        const ReadFields fields{};
         // the wetting wall's solid plane and a frozen temperature are separate instantiations (FP32 storage
         // only), so that the kernel without them carries no trace of them
 #define GB300_TMA_CASE(I, X, Y)                                                                                \
         case I:                                                                                                \
-            if (precision == 0 && P.thermal_off && P.wet) GB300_TMA(X, Y, float, true, true)                   \
-            else if (precision == 0 && P.thermal_off) GB300_TMA(X, Y, float, false, true)                      \
-            else if (precision == 0 && P.wet) GB300_TMA(X, Y, float, true, false)                              \
-            else if (precision == 0) GB300_TMA(X, Y, float, false, false)                                      \
-            else if (precision == 1) GB300_TMA(X, Y, __nv_bfloat16, false, false)                              \
-            else GB300_TMA(X, Y, __half, false, false)                                                         \
+            if (precision == 0 && P.thermal_off && P.wet) GB300_TMA(X, Y, float, true, true, false)                   \
+            else if (precision == 0 && P.thermal_off) GB300_TMA(X, Y, float, false, true, false)                      \
+            else if (precision == 0 && P.wet) GB300_TMA(X, Y, float, true, false, false)                              \
+            else if (precision == 0) GB300_TMA(X, Y, float, false, false, false)                                      \
+            else if (precision == 1) GB300_TMA(X, Y, __nv_bfloat16, false, false, false)                              \
+            else GB300_TMA(X, Y, __half, false, false, false)                                                         \
             break;
         switch (maps->shape) {
             GB300_TMA_SHAPES(GB300_TMA_CASE)
         default: return cudaErrorInvalidValue;
         }
 #undef GB300_TMA_CASE
-#undef GB300_TMA
         return cudaGetLastError();
     }
     const int zc = zchunk_generic(P, tiles_x * tiles_y);
@@ -1468,13 +1516,29 @@ static int zchunk_readout(const DevParams& P, long long tiles) {
 }
 
 cudaError_t launch_readout(const DevParams& P, int precision, const StateBufs& B, const double* sums_cur, float* rho,
-                           float* ux, float* uy, float* uz, float* T, cudaStream_t s) {
+                           float* ux, float* uy, float* uz, float* T, cudaStream_t s, const TmaMaps* maps) {
+    // The TMA kernel's read-out instantiation (maps of kReadShape) where its copies pay: from 2^17 nodes
+    // (32^3 24 us a call against k_readout's 22, 64 x 64 x 96 33 against 39, 200 x 200 x 300 369 against 527), and
+    // not for a frozen g, whose planes z - 1 and z + 1 it would fetch for nothing (181 against 174).
+    if (maps && maps->ok && P.N >= 1 << 17 && !P.thermal_off && tma_runs(P, precision, B)) {
+        constexpr int TXR = kTmaTX[kReadShape], TYR = kTmaTY[kReadShape];
+        const int txs = (P.nx + TXR - 1) / TXR, tys = (P.ny + TYR - 1) / TYR;
+        const int ctas = maps->sms < maps->items ? maps->sms : maps->items, first = 0;
+        double* sums_next = nullptr;
+        const ReadFields fields{rho, ux, uy, uz, T};
+        cudaError_t e = cudaSuccess;
+        if (precision == 0 && P.wet) GB300_TMA(TXR, TYR, float, true, false, true)
+        else if (precision == 0) GB300_TMA(TXR, TYR, float, false, false, true)
+        else if (precision == 1) GB300_TMA(TXR, TYR, __nv_bfloat16, false, false, true)
+        else GB300_TMA(TXR, TYR, __half, false, false, true)
+        return cudaGetLastError();
+    }
     const int tiles_x = (P.nx + TX - 1) / TX, tiles_y = (P.ny + kTY - 1) / kTY;
     const int zc = zchunk_readout(P, (long long)tiles_x * tiles_y);
     const dim3 grid(tiles_x, tiles_y, (P.nz + zc - 1) / zc);
 #define GB300_READ(S, QT)                                                                                      \
     k_readout<S, QT, false, false><<<grid, FusedShape<kTY, QT>::kThreads, 0, s>>>(                             \
-        P, nullptr, nullptr, (const S*)B.src, B.pull_f, B.pull_g, sums_cur, zc, rho, ux, uy, uz, T, B.flag,    \
+        P, nullptr, nullptr, (const S*)B.src, B.pull_f, B.pull_g, sums_cur, zc, ReadFields{rho, ux, uy, uz, T}, B.flag,    \
         nullptr, nullptr, nullptr, nullptr, nullptr)
     if (P.qt == 19) {
         if (precision != 0) return cudaErrorInvalidValue;
@@ -1498,8 +1562,8 @@ cudaError_t launch_psi_velocity(const DevParams& P, int precision, const StateBu
     const dim3 grid(tiles_x, tiles_y, (P.nz + zc - 1) / zc);
 #define GB300_VEL(S, QT)                                                                                       \
     k_readout<S, QT, false, true><<<grid, FusedShape<kTY, QT>::kThreads, 0, s>>>(                              \
-        P, nullptr, nullptr, (const S*)B.src, B.pull_f, B.pull_g, sums_cur, zc, nullptr, nullptr, nullptr, nullptr, \
-        nullptr, B.flag, B.psirho, B.vel, B.partial, B.counter, sums)
+        P, nullptr, nullptr, (const S*)B.src, B.pull_f, B.pull_g, sums_cur, zc, ReadFields{}, B.flag,     \
+        B.psirho, B.vel, B.partial, B.counter, sums)
     if (P.qt == 19) {
         if (precision != 0) return cudaErrorInvalidValue;
         GB300_VEL(float, 19);
@@ -1520,7 +1584,7 @@ cudaError_t launch_readout_batch(const DevParams& P, int precision, const BatchI
                                  float* uy, float* uz, float* T, cudaStream_t s) {
 #define GB300_READ(S)                                                                                          \
     k_readout<S, 7, true, false><<<n_items, FusedShape<kTY>::kThreads, 0, s>>>(                                \
-        P, insts, items, (const S*)B.src, B.pull_f, B.pull_g, sums_cur, 0, rho, ux, uy, uz, T, B.flag, nullptr, \
+        P, insts, items, (const S*)B.src, B.pull_f, B.pull_g, sums_cur, 0, ReadFields{rho, ux, uy, uz, T}, B.flag, nullptr, \
         nullptr, nullptr, nullptr, nullptr)
     switch (precision) {
     case 0: GB300_READ(float); break;

@@ -106,9 +106,11 @@ int tma_ghost_cols(int precision);
 int tma_tile_h(int shape);
 
 // macroscopic fields of the current state (B.src) into the device arrays given (each nullable); a
-// scheme-1 wetting wall's table must be that of this state
+// scheme-1 wetting wall's table must be that of this state.  With maps (of tile shape tma_read_shape())
+// and a state the TMA kernel reads, its read-out instantiation runs, else k_readout.
 cudaError_t launch_readout(const DevParams& P, int precision, const StateBufs& B, const double* sums_cur, float* rho,
-                           float* ux, float* uy, float* uz, float* T, cudaStream_t s);
+                           float* ux, float* uy, float* uz, float* T, cudaStream_t s, const TmaMaps* maps);
+int tma_read_shape();
 
 // deterministic FP64 sum of a float field into out[0] (out[1] = 0).
 cudaError_t launch_sum_field(const float* a, int n, double2* partial, unsigned* counter,
