@@ -98,7 +98,7 @@ typedef struct {
     void* workspace;              /* optional caller-owned device memory (see above) */
     size_t workspace_bytes;
     int test_stall;               /* test of the timeout path only (0 in normal use): in the next
-                                     step of the TMA kernel the producer waits for its first stage
+                                     step of the TMA kernel the copy warp waits for its first stage
                                      to be released before loading it, which nothing can do, so
                                      the bounded waits give up and lbm_step reports LBM_ETIMEOUT;
                                      cleared once that step is enqueued (never graph-captured) */

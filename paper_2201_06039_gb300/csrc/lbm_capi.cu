@@ -429,6 +429,61 @@ int check_flag(lbm_ctx* c) {
 
 }  // namespace
 
+namespace {
+
+EncodeTiledFn tensor_map_encoder() {   // looked up once a process (a lookup takes tens of microseconds)
+    static const EncodeTiledFn fn = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return (EncodeTiledFn)f;
+    }();
+    return fn;
+}
+
+CUtensorMapDataType map_type(int precision) {
+    return precision == LBM_FP32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
+         : precision == LBM_BF16_SHIFTED ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
+}
+
+// the two load maps (14- and 6-slot windows of a tile shape) of population buffer k
+bool encode_loads(EncodeTiledFn encode, const DevParams& d, int precision, void* buf, int shape, int k, TmaMaps* maps) {
+    const cuuint64_t E = (cuuint64_t)pop_bytes(precision);
+    const cuuint64_t dims[4] = {(cuuint64_t)d.Ws, (cuuint64_t)d.Hs, (cuuint64_t)d.nz, (cuuint64_t)kSlots};
+    const cuuint64_t strides[3] = {(cuuint64_t)d.Rs * E, (cuuint64_t)d.splane * E, (cuuint64_t)d.Ns * E};
+    const cuuint32_t bw = (cuuint32_t)tma_box_w(shape, precision), bh = (cuuint32_t)tma_box_h(shape);
+    const cuuint32_t box14[4] = {bw, bh, 1, 14}, box6[4] = {bw, bh, 1, 6}, es[4] = {1, 1, 1, 1};
+    return encode(&maps->m14[k], map_type(precision), 4, buf, dims, strides, box14, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS &&
+           encode(&maps->m6[k], map_type(precision), 4, buf, dims, strides, box6, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+}  // namespace
+
+bool gb300lbm::build_read_maps(const DevParams& d, int precision, void* buf0, void* buf1, const TmaMaps& step,
+                               TmaMaps* maps) {
+    *maps = step;
+    maps->ok = false;
+    int shape = -1, zchunk = 0, items = 0;
+    tma_plan_for(d, step.sms, tma_read_shape(), 0, 1 << 30, &shape, &zchunk, &items);
+    if (!step.ok || shape < 0) return false;
+    maps->shape = shape;
+    maps->zchunk = zchunk;
+    maps->items = items;
+    if (shape != step.shape)
+        for (int k = 0; k < 2; ++k)
+            if (!encode_loads(tensor_map_encoder(), d, precision, k == 0 ? buf0 : buf1, shape, k, maps)) return false;
+    maps->ok = true;
+    return true;
+}
+
 bool gb300lbm::build_tma_maps(const DevParams& d, int precision, void* buf0, void* buf1, int model_ctas,
                               int forced_shape, int forced_zchunk, int max_items, TmaMaps* maps) {
     maps->ok = false;
@@ -440,22 +495,11 @@ bool gb300lbm::build_tma_maps(const DevParams& d, int precision, void* buf0, voi
     int shape = -1, zchunk = 0, items = 0;
     tma_plan_for(d, model_ctas > 0 ? model_ctas : sms, forced_shape, forced_zchunk, max_items, &shape, &zchunk, &items);
     if (shape < 0 || (size_t)optin < tma_smem_bytes(shape, precision)) return false;
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess || !fn) {
-        cudaGetLastError();
-        return false;
-    }
-    EncodeTiledFn encode = (EncodeTiledFn)fn;
-    cuuint64_t dims[4] = {(cuuint64_t)d.Ws, (cuuint64_t)d.Hs, (cuuint64_t)d.nz, (cuuint64_t)kSlots};
+    const EncodeTiledFn encode = tensor_map_encoder();
+    if (!encode) return false;
     const cuuint64_t E = (cuuint64_t)pop_bytes(precision);
-    const CUtensorMapDataType dt = precision == LBM_FP32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
-                                 : precision == LBM_BF16_SHIFTED ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
-                                                                      : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
-    cuuint64_t strides[3] = {(cuuint64_t)d.Rs * E, (cuuint64_t)d.splane * E, (cuuint64_t)d.Ns * E};
-    const cuuint32_t bw = (cuuint32_t)tma_box_w(shape, precision), bh = (cuuint32_t)tma_box_h(shape);
-    cuuint32_t box14[4] = {bw, bh, 1, 14}, box6[4] = {bw, bh, 1, 6}, es[4] = {1, 1, 1, 1};
+    const CUtensorMapDataType dt = map_type(precision);
+    const cuuint32_t es[4] = {1, 1, 1, 1};
     // output tiles, dimensions ordered (x, slot, y, z) to match the [row][slot][x] out buffer; the
     // tensor spans the real nodes only (x < nx, y < ny in storage coordinates + the offsets), and
     // the last tile row gets a box of exactly its rows, so no box ever extends past ny
@@ -476,14 +520,7 @@ bool gb300lbm::build_tma_maps(const DevParams& d, int precision, void* buf0, voi
     maps->ghosts = tma_ghost_mode(d, shape, precision);
     for (int k = 0; k < 2; ++k) {
         void* g = k == 0 ? buf0 : buf1;
-        if (encode(&maps->m14[k], dt, 4, g, dims, strides, box14, es,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return false;
-        if (encode(&maps->m6[k], dt, 4, g, dims, strides, box6, es,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return false;
+        if (!encode_loads(encode, d, precision, g, shape, k, maps)) return false;
         if (encode(&maps->mout[k], dt, 4, g, dims_out, strides_out, box_out, es,
                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
@@ -593,7 +630,7 @@ int lbm_create(const lbm_params* p, lbm_ctx** out) {
     c->plan_zchunk = 0;
     c->dp.check_flag = (int*)(c->base + c->L.flag);
     if (c->variant == LBM_KERNEL_FUSED && p->use_tma != 0 && make_tma_maps(c))
-        build_tma_maps(c->dp, c->p.precision, c->pbuf(0), c->pbuf(1), 0, tma_read_shape(), 0, max_partials(c->dp), &c->read_maps);
+        build_read_maps(c->dp, c->p.precision, c->pbuf(0), c->pbuf(1), c->maps, &c->read_maps);
     cudaError_t e = cudaMemsetAsync(c->base + c->L.sums, 0, c->L.flag + sizeof(int) - c->L.sums, c->stream);
     if (e == cudaSuccess && c->dp.wet) {   // scheme 0: the table is constant; scheme 1: refreshed every step
         c->dp.wall_tab = (const float2*)(c->base + c->L.wall);

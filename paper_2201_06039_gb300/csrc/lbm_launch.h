@@ -72,6 +72,10 @@ struct TmaMaps {
 bool build_tma_maps(const DevParams& d, int precision, void* buf0, void* buf1, int model_ctas, int forced_shape,
                     int forced_zchunk, int max_items, TmaMaps* maps);
 
+// Load maps and plan of the read-out (tile shape tma_read_shape(), no partial sums) beside the step's
+// maps of the same lattice and buffers.
+bool build_read_maps(const DevParams& d, int precision, void* buf0, void* buf1, const TmaMaps& step, TmaMaps* maps);
+
 // fused z-marching variant (psi of the tile halo recomputed from the populations); uses the
 // TMA kernel when maps are given and the lattice / state qualify (see tma_eligible).
 // *ghosts_written (nullable) tells whether the launch also refreshed the ghost cells of dst.
@@ -86,8 +90,8 @@ bool tma_eligible(const DevParams& P, int precision);
 bool tma_runs(const DevParams& P, int precision, const StateBufs& B);
 // refresh the ghost columns / rows of a population buffer from their periodic images
 cudaError_t launch_ghosts(const DevParams& P, int precision, void* pops, cudaStream_t s);
-// tile shapes 0: 32 x 8, 1: 40 x 7, 2: 32 x 12, 3: 24 x 16 (window boxes tma_box_w x tma_box_h per
-// population slot)
+// tile shapes 0: 32 x 8, 1: 40 x 7, 2: 32 x 12, 3: 24 x 16, 4: 40 x 8, 5: 40 x 10 (window boxes tma_box_w x
+// tma_box_h per population slot)
 // forced_shape >= 0 / forced_zchunk > 0 pin the shape / the z-chunk of the plan; plans of more than
 // max_items items are not considered (*shape -1 if none is left)
 void tma_plan_for(const DevParams& P, int ctas, int forced_shape, int forced_zchunk, int max_items, int* shape,
