@@ -644,13 +644,16 @@ __device__ __forceinline__ void load_g19(const DevParams& P, const S* __restrict
     }
 }
 
-// the 19 f and 19 g of a node at storage index i (FP32 storage only)
+// the 19 f, and the 19 g, of a node at storage index i (FP32 storage only)
 template <typename S>
-__device__ __forceinline__ void store_slots19(const DevParams& P, S* __restrict__ dst, int i, const float f[19],
-                                              const float g[19]) {
+__device__ __forceinline__ void store_f(const DevParams& P, S* __restrict__ dst, int i, const float f[19]) {
     S* q = dst + bidx(P, i, P.Nidx);
 #pragma unroll
     for (int a = 0; a < 19; ++a) Codec<S>::store(q + (size_t)fslot(a) * P.Ns, f[a], 0.f);
+}
+template <typename S>
+__device__ __forceinline__ void store_g19(const DevParams& P, S* __restrict__ dst, int i, const float g[19]) {
+    S* q = dst + bidx(P, i, P.Nidx);
 #pragma unroll
     for (int a = 0; a < 19; ++a) Codec<S>::store(q + (size_t)gslot19(a) * P.Ns, g[a], 0.f);
 }
@@ -741,7 +744,8 @@ template <> struct Therm<19> {
     template <typename S>
     static __device__ __forceinline__ void store(const DevParams& P, S* dst, int i, const float f[19],
                                                  const float g[19]) {
-        store_slots19<S>(P, dst, i, f, g);
+        store_f<S>(P, dst, i, f);
+        store_g19<S>(P, dst, i, g);
     }
     static __device__ __forceinline__ void equilibrium(const DevParams&, float T, float g[19]) {
 #pragma unroll

@@ -16,10 +16,11 @@
 // k_fused_tma : FP32 or shifted 16-bit storage, any faces, g evolving (or frozen, FP32).  A
 //               copy warp fetches each plane's pulls for the whole tile + halo with three TMA
 //               tensor copies (one per e_z group of population slots) into a multi-stage
-//               shared-memory pipeline guarded by mbarriers; psi warps and collision warps read
-//               every pull as one shared-memory load at a fixed offset.  FP32 planes leave through
-//               TMA tensor stores, 16-bit planes through direct stores of the collision threads.
-//               Persistent CTAs take (z-chunk, tile) items round robin.
+//               shared-memory pipeline guarded by mbarriers; compute and halo warps read every
+//               pull as one shared-memory load at a fixed offset, and collided planes leave
+//               through TMA tensor stores.  Persistent CTAs take (z-chunk, tile) items round
+//               robin.
+// k_readout   : macroscopic fields (and the first pass of a finite-difference div u step).
 #include <cuda.h>
 
 #include <algorithm>
@@ -199,15 +200,23 @@ __device__ __forceinline__ void fused_column(const DevParams& P, const S* __rest
         const int i = sidx(P, mx, my, mz);
         Nbr n = make_nbr(P, mx, my, mz);
         float f[19], g[QT];
+        float* st = stage + ((zp - z0) & 1) * Sh::kStageFloats + tid;
         load_f<S>(P, src, pull_f, i, mx, my, mz, n, f);
+        const float rho = sum19(f);
+        if (QT != 7 && owner && in_chunk) {   // f is put away before g is pulled
+#pragma unroll
+            for (int a = 0; a < 19; ++a) st[a * Sh::kInterior] = f[a];
+        }
+        if (QT != 7) asm volatile("" ::: "memory");
         Therm<QT>::template load<S>(P, src, pull_g, i, mx, my, mz, n, g);
-        float rho = sum19(f), T = Therm<QT>::sum(g);
+        const float T = Therm<QT>::sum(g);
         float psi2 = psi_squared(P, rho, T);
         ring[((zp + 4) % Sh::kRing) * Sh::kRingPlane + slot] = make_float2(psi_of(psi2), rho);
         if (owner && in_chunk) {
-            float* st = stage + ((zp - z0) & 1) * Sh::kStageFloats + tid;
+            if (QT == 7) {
 #pragma unroll
-            for (int a = 0; a < 19; ++a) st[a * Sh::kInterior] = f[a];
+                for (int a = 0; a < 19; ++a) st[a * Sh::kInterior] = f[a];
+            }
 #pragma unroll
             for (int a = 0; a < QT; ++a) st[(19 + a) * Sh::kInterior] = g[a];
             kahan_add(r_sum, r_c, rho);
@@ -224,9 +233,12 @@ __device__ __forceinline__ void fused_column(const DevParams& P, const S* __rest
         float f[19], g[QT];
 #pragma unroll
         for (int a = 0; a < 19; ++a) f[a] = st[a * Sh::kInterior];
+        auto load_staged_g = [&] {
 #pragma unroll
-        for (int a = 0; a < QT; ++a) g[a] = st[(19 + a) * Sh::kInterior];
-        float rho = sum19(f), T = Therm<QT>::sum(g);
+            for (int a = 0; a < QT; ++a) g[a] = st[(19 + a) * Sh::kInterior];
+        };
+        if constexpr (QT == 7) load_staged_g();
+        float rho = sum19(f);
         const float2* rm = ring + ((z + 3) % Sh::kRing) * Sh::kRingPlane;
         const float2* r0 = ring + (z % Sh::kRing) * Sh::kRingPlane;
         const float2* rp = ring + ((z + 1) % Sh::kRing) * Sh::kRingPlane;
@@ -235,15 +247,21 @@ __device__ __forceinline__ void fused_column(const DevParams& P, const S* __rest
                                       Sh::kRingW);
         const Forces F = total_force(P, me.x, rs.Fx, rs.Fy, rs.Fz, rho - rho_ave);
         NodeOut o = collide_f(P, f, rho, F.Fx, F.Fy, F.Fz, F.Fm2, me.x * me.x);
-        float ph = Therm<QT>::collide(P, g, rho, T, o, rs.gx, rs.gy, rs.gz, phis[d], first);
         // frozen fields keep their stored values (no streaming, no collision)
         if (P.flow_off) {
 #pragma unroll
             for (int a = 0; a < 19; ++a)
                 f[a] = Codec<S>::load(src + (size_t)fslot(a) * P.Ns + bidx(P, i, P.Nidx), P.shift_f[a]);
         }
+        if constexpr (QT != 7) {   // f leaves before g is taken up: 38 populations at once spill
+            store_f<S>(P, dst, i, f);
+            load_staged_g();
+        }
+        const float T = Therm<QT>::sum(g);
+        float ph = Therm<QT>::collide(P, g, rho, T, o, rs.gx, rs.gy, rs.gz, phis[d], first);
         if (P.thermal_off) Therm<QT>::template stored<S>(P, src, i, g);
-        Therm<QT>::template store<S>(P, dst, i, f, g);
+        if constexpr (QT == 7) Therm<QT>::template store<S>(P, dst, i, f, g);
+        else store_g19<S>(P, dst, i, g);
         phis[d] = ph;
     };
 
@@ -494,7 +512,7 @@ k_readout(DevParams P0, const BatchInst* __restrict__ insts, const BatchItem* __
     }
 }
 
-// ================================================================ TMA producer / consumer kernel
+// ================================================================ TMA kernel
 // Tile TX x TY.  Warps: copy warp (TMA loads and stores), compute warps (one tile node per thread:
 // pull, psi, collision), two halo warps (psi of the one-node ring around the tile).
 constexpr size_t align128(size_t v) { return (v + 127) / 128 * 128; }
@@ -1005,7 +1023,7 @@ k_fused_tma(const __grid_constant__ CUtensorMap map14, const __grid_constant__ C
             const bool hx = ghosts == 2 && owner && (gx < 2 || gx >= P.nx - 2);
             const bool hy = ghosts == 2 && owner && (gy < 2 || gy >= P.ny - 2);
             const int ix = gx < 2 ? gx + P.nx : gx - P.nx, iy = gy < 2 ? gy + P.ny : gy - P.ny;
-            // ... and the last tile column of such a lattice stores its nodes directly (see storer)
+            // ... and the last tile column of such a lattice stores its nodes directly (see the copy warp)
             const bool direct_tile = ghosts == 2 && x0 + TX_ > P.nx && P.nx % kGW != 0;
             const int cx4 = !owner ? -1 : eright ? (gx >= P.nx - kGW ? gx - (P.nx - kGW) : -1)
                                         : eleft ? (gx < kGW ? gx : -1) : -1;
