@@ -6,7 +6,6 @@
 //             slots layout of a single lattice, so the per-instance set-up and read-out kernels
 //             run unchanged on the instance's block)
 //   phis      phi_s history, instances concatenated (node offset field_off_k)
-//   psirho    (psi, rho) scratch of the largest instance (totals only)
 //   sums      (sum rho, sum T) per instance: two ping-pong sets (rho_ave of the next step) and
 //             one set for lbm_batch_get_totals
 //   partial   one double2 per work item (and per block of the read-out reductions)
@@ -68,10 +67,10 @@ struct lbm_batch {
     std::vector<int> order;            // instances by size, largest first
     long long nodes;                   // total nodes
     long long pop_elems;               // elements of one population buffer
-    int max_N, max_items, max_partial;
+    int max_items, max_partial;
     cudaStream_t stream, capture, launch;
     char* base;
-    size_t off_pops[2], off_phis, off_psirho, off_sums, off_partial, off_counters, off_flag, off_inst, off_items, off_ritems;
+    size_t off_pops[2], off_phis, off_sums, off_partial, off_counters, off_flag, off_inst, off_items, off_ritems;
     int plan, n_items, ctas, sms;
     int n_ritems;                      // items of the read-out table
     int cur, slot;
@@ -108,7 +107,7 @@ struct lbm_batch {
         B.src_index = cur;
         B.pull_f = fresh_f ? 0 : 1;
         B.pull_g = fresh_g ? 0 : 1;
-        B.psirho = (float2*)(base + off_psirho);
+        B.psirho = nullptr;
         B.phis = phis() + fo;
         B.partial = (double2*)(base + off_partial);
         B.counter = k < 0 ? counters() : counters() + 2;
@@ -429,7 +428,6 @@ int lbm_batch_create(const lbm_params* common, int n_instances, const int* dims,
     b->inst.resize(n_instances);
     b->nodes = 0;
     b->pop_elems = 0;
-    b->max_N = 0;
     for (int k = 0; k < n_instances; ++k) {
         lbm_params pk = *common;
         pk.nx = dims[3 * k];
@@ -452,7 +450,6 @@ int lbm_batch_create(const lbm_params* common, int n_instances, const int* dims,
         I.inv_N = d.inv_N;
         b->pop_elems += (long long)pop_elems(d);
         b->nodes += d.N;
-        b->max_N = std::max(b->max_N, d.N);
     }
     if (b->nodes >= (1LL << 40)) {
         delete b;
@@ -488,7 +485,6 @@ int lbm_batch_create(const lbm_params* common, int n_instances, const int* dims,
     b->off_pops[0] = take((size_t)b->pop_elems * pb);
     b->off_pops[1] = take((size_t)b->pop_elems * pb);
     b->off_phis = take(4 * (size_t)b->nodes);
-    b->off_psirho = take(8 * (size_t)b->max_N);
     b->off_sums = take(sizeof(double) * 6 * (size_t)n_instances);
     b->off_partial = take(sizeof(double2) * (size_t)b->max_partial);
     b->off_counters = take((4 + (size_t)n_instances) * sizeof(unsigned));
@@ -520,8 +516,9 @@ int lbm_batch_create(const lbm_params* common, int n_instances, const int* dims,
     }
     for (auto& d : b->dps) d.check_flag = (int*)(b->base + b->off_flag);
     e = cudaMemsetAsync(b->base + b->off_sums, 0, b->off_inst - b->off_sums, b->stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(b->d_ritems(), ritems.data(), sizeof(BatchItem) * ritems.size(), cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
-    if (e == cudaSuccess) e = cudaMemcpy(b->d_ritems(), ritems.data(), sizeof(BatchItem) * ritems.size(), cudaMemcpyHostToDevice);
     int rc = e == cudaSuccess ? set_plan(b, 0) : fail(LBM_ECUDA, "initial memset: %s", cudaGetErrorString(e));
     if (rc) {
         cudaFree(b->base);
@@ -714,7 +711,6 @@ int lbm_batch_get_totals(lbm_batch* b, double* sums) {
     if (!b->initialised) return fail(LBM_ESTATE, "lbm_batch_get_totals before lbm_batch_init_fields");
     for (int k = 0; k < b->n; ++k) {
         StateBufs B = b->bufs(k);
-        B.psirho = nullptr;   // sums only
         GB300_CK(launch_psi(b->dps[k], b->p.precision, B, b->sums(2) + 2 * k, b->stream));
     }
     GB300_CK(cudaMemcpyAsync(sums, b->sums(2), sizeof(double) * 2 * b->n, cudaMemcpyDeviceToHost, b->stream));
