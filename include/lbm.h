@@ -290,7 +290,7 @@ long long lbm_batch_nodes(const lbm_batch* b, int instance);
 int lbm_batch_init_fields(lbm_batch* b, const float* rho, const float* T, const float* u);
 int lbm_batch_step(lbm_batch* b, int n);
 /* Time every candidate work plan (tile rows 4 or 8, columns split into 1, 2 or 4 z-chunks, and
- * the TMA mode) over `steps` steps of the current state, keep the fastest, and restore the state exactly
+ * the TMA mode, this one over 8 steps) over `steps` steps of the current state, keep the fastest, and restore the state exactly
  * (the candidates' steps are undone).  Needs free device memory for one copy of the state.
  * best_ms (nullable) receives the chosen plan's time per step. */
 int lbm_batch_autotune(lbm_batch* b, int steps, double* best_ms);
