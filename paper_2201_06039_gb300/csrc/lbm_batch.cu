@@ -52,7 +52,7 @@ const int kTmaChain = 8;                                            // steps of 
 
 struct BatchGraph {
     int n, cur, slot, plan;
-    bool ghosts_valid;
+    bool ghosts_valid, fresh_f, fresh_g;   // form of the state (see GraphEntry of the single lattice)
     cudaGraphExec_t exec;
 };
 const int kBatchGraphs = 4;
@@ -326,7 +326,8 @@ int batch_graph(lbm_batch* b, int m, cudaGraphExec_t* out) {
     BatchGraph* hit = nullptr;
     for (int k = 0; k < b->n_graphs; ++k) {
         BatchGraph& g = b->graphs[k];
-        if (g.n == m && g.cur == b->cur && g.slot == b->slot && g.plan == b->plan && g.ghosts_valid == b->ghosts_valid)
+        if (g.n == m && g.cur == b->cur && g.slot == b->slot && g.plan == b->plan && g.ghosts_valid == b->ghosts_valid &&
+            g.fresh_f == b->fresh_f && g.fresh_g == b->fresh_g)
             hit = &g;
     }
     if (!hit) {
@@ -358,6 +359,7 @@ int batch_graph(lbm_batch* b, int m, cudaGraphExec_t* out) {
         }
         BatchGraph& g = b->graphs[b->n_graphs++];
         g.n = m; g.cur = b->cur; g.slot = b->slot; g.plan = b->plan; g.ghosts_valid = b->ghosts_valid; g.exec = exec;
+        g.fresh_f = b->fresh_f; g.fresh_g = b->fresh_g;
         hit = &g;
     }
     *out = hit->exec;

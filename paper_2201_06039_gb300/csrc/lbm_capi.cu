@@ -73,8 +73,13 @@ Layout layout_of(const lbm_params* p, const DevParams& dp) {
 
 const int kGraphCache = 8;
 
+// A captured run of n steps: what it holds, beyond the buffers, maps and parameters of the context, is
+// where it starts (cur, slot) and the form of the state (fresh_f, fresh_g: they give each launch its
+// pull flags and choose the kernel).  A frozen field keeps its form, which differs between
+// lbm_init_fields and a loaded checkpoint of a run in which it evolved.
 struct GraphEntry {
     int n, cur, slot;
+    bool fresh_f, fresh_g;
     cudaGraphExec_t exec;
     unsigned long long last_use;
 };
@@ -367,7 +372,8 @@ int run_graph(lbm_ctx* c, int n) {
     GraphEntry* hit = nullptr;
     for (int k = 0; k < c->n_graphs; ++k) {
         GraphEntry& g = c->graphs[k];
-        if (g.n == n && g.cur == c->cur && g.slot == c->slot) hit = &g;
+        if (g.n == n && g.cur == c->cur && g.slot == c->slot && g.fresh_f == c->fresh_f && g.fresh_g == c->fresh_g)
+            hit = &g;
     }
     if (!hit) {
         int c0 = c->cur, s0 = c->slot;
@@ -400,6 +406,7 @@ int run_graph(lbm_ctx* c, int n) {
         }
         GraphEntry& g = c->graphs[c->n_graphs++];
         g.n = n; g.cur = c->cur; g.slot = c->slot; g.exec = exec;
+        g.fresh_f = c->fresh_f; g.fresh_g = c->fresh_g;
         hit = &g;
     }
     hit->last_use = ++c->use_clock;
@@ -671,7 +678,8 @@ int lbm_init_fields(lbm_ctx* c, const float* rho, const float* T, const float* u
         CK(cudaMemcpyAsync(stage + 2 * N, u, 3 * N * 4, cudaMemcpyHostToDevice, c->stream));
         du = stage + 2 * N;
     }
-    // (captured step graphs stay: they hold the buffers, maps and parameters, which do not change here)
+    // (captured step graphs stay: buffers, maps and parameters do not change here, and run_graph
+    // replays one only for a state of the form it was captured for)
     c->cur = 0;
     c->slot = 0;
     CK(launch_init(c->dp, c->p.precision, c->pbuf(0), drho, dT, du, c->stream));
