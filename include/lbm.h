@@ -101,7 +101,9 @@ typedef struct {
                                      step of the TMA kernel the copy warp waits for its first stage
                                      to be released before loading it, which nothing can do, so
                                      the bounded waits give up and lbm_step reports LBM_ETIMEOUT;
-                                     cleared once that step is enqueued (never graph-captured) */
+                                     cleared once that step is enqueued (never graph-captured).
+                                     2: the same in the next read-out that runs on the TMA kernel
+                                     (lbm_get_moments reports LBM_ETIMEOUT) */
     int thermal_bgk;              /* 1: single-relaxation-time (BGK) D3Q7 collision, every
                                      non-conserved moment relaxed at 1/varsigma_T, in place of
                                      the free rates varsigma_q, varsigma_pi of Eq. 43 (MRT) */
@@ -169,8 +171,11 @@ int lbm_step(lbm_ctx* ctx, int n);
 
 /* Macroscopic fields of the current state: rho = sum f (Eq. 10), u = (sum e f + F/2)/rho
  * (Eq. 10, F = F_m of Eq. 7 + F_b with the rho_ave the next step uses), T = sum g (Eq. 20).
- * Any output pointer may be NULL.  Synchronises the stream before returning.
- * Errors: LBM_ESTATE, LBM_ECUDA. */
+ * Any output pointer may be NULL.  Synchronises the stream before returning.  Where the read-out runs
+ * on the TMA kernel its waits are bounded: LBM_ETIMEOUT if one gave up, in this call or in earlier steps
+ * that did not report it (check_nonfinite 0).  The fields are then not valid; after a wait of the read-out
+ * itself the state is as before and the call can be made again.
+ * Errors: LBM_ESTATE, LBM_ECUDA, LBM_ETIMEOUT. */
 int lbm_get_moments(lbm_ctx* ctx, float* rho, float* ux, float* uy, float* uz, float* T);
 
 /* FP64 totals of the current state, reduced deterministically on the device:

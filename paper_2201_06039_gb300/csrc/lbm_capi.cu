@@ -230,7 +230,7 @@ DevParams make_dev(const lbm_params* p) {
     d.rho_buoy = p->rho_buoy > 0.0 ? (float)p->rho_buoy : 0.f;
     d.flow_off = p->flow_off; d.thermal_off = p->thermal_off;
     d.qt = p->thermal_q == 19 ? 19 : 7;
-    d.test_stall = p->test_stall ? 1 : 0;
+    d.test_stall = p->test_stall == 2 ? 2 : p->test_stall ? 1 : 0;
     d.thermal_bgk = p->thermal_bgk ? 1 : 0;
     d.divu_mode = p->divu_mode;
     d.wet = (p->wall_rho > 0.0 || p->wall_scheme == 1) && p->bc[4] == LBM_BC_WALL ? 1 : 0;
@@ -335,7 +335,7 @@ int enqueue_step(lbm_ctx* c, KernelTimer* timer = nullptr) {
         e = launch_fused(c->dp, c->p.precision, B, c->sums(c->slot), c->sums(c->slot ^ 1), c->first ? 1 : 0,
                          c->launch, c->maps.ok ? &c->maps : nullptr, &ghosts_done);
         if (e != cudaSuccess) return fail(LBM_ECUDA, "fused kernel launch: %s", cudaGetErrorString(e));
-        if (c->maps.ok && tma_runs(c->dp, c->p.precision, B)) c->dp.test_stall = 0;   // one stalled TMA step only
+        if (c->dp.test_stall == 1 && c->maps.ok && tma_runs(c->dp, c->p.precision, B)) c->dp.test_stall = 0;   // one step only
         if (timer) timer->end(0, c->launch);
     } else {
         if (timer) timer->begin(c->launch);
@@ -709,7 +709,7 @@ int lbm_step(lbm_ctx* c, int n) {
         ++k;
     }
     if (k < n) {
-        if (c->p.use_graph && !c->dp.test_stall) rc = run_graph(c, n - k);   // never capture a stall
+        if (c->p.use_graph && c->dp.test_stall != 1) rc = run_graph(c, n - k);   // never capture a stall
         else
             for (; k < n && rc == LBM_OK; ++k) rc = enqueue_step(c);
         if (rc) return rc;
@@ -748,12 +748,21 @@ int lbm_get_moments(lbm_ctx* c, float* rho, float* ux, float* uy, float* uz, flo
     float* outs[5] = {rho, ux, uy, uz, T};
     float* dst[5];
     for (int k = 0; k < 5; ++k) dst[k] = outs[k] ? (is_device_ptr(outs[k]) ? outs[k] : stage + k * N) : nullptr;
+    bool bounded_waits = false;
     CK(launch_readout(c->dp, c->p.precision, B, c->sums(c->slot), dst[0], dst[1], dst[2], dst[3], dst[4], c->stream,
-                      c->maps.ok ? &c->read_maps : nullptr));
+                      c->maps.ok ? &c->read_maps : nullptr, &bounded_waits));
+    if (bounded_waits && c->dp.test_stall == 2) c->dp.test_stall = 0;   // one stalled read-out only
+    int flag = 0;
+    if (bounded_waits)
+        CK(cudaMemcpyAsync(&flag, c->base + c->L.flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     for (int k = 0; k < 5; ++k)
         if (outs[k] && dst[k] != outs[k])
             CK(cudaMemcpyAsync(outs[k], dst[k], N * 4, cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
+    if (flag & 2) {   // reported here; the flag word's other bits (its low byte) stay for lbm_step
+        CK(cudaMemsetAsync(c->base + c->L.flag, flag & ~2, 1, c->stream));
+        return fail(LBM_ETIMEOUT, "a bounded pipeline wait gave up: the fields are not valid (step %lld)", c->steps);
+    }
     return LBM_OK;
 }
 

@@ -79,7 +79,7 @@ struct DevParams {
     float gx, gy, gz;
     float rho_buoy;           // > 0: fixed reference density of the buoyancy force, else rho_ave
     int flow_off, thermal_off;
-    int test_stall;           // timeout-path test: the TMA producer waits on a barrier nothing completes
+    int test_stall;           // timeout-path test: the copy warp of the next TMA step (1) or read-out (2) waits on a barrier nothing completes
     int thermal_bgk;          // 1: BGK D3Q7 collision (n4..n6 relaxed at 1/varsigma_T too)
     int divu_mode;            // 1: finite-difference div u away from solid faces (two-pass kernels)
     int wet;                  // 1: virtual-density solid layer below the -z wall (wetting)

@@ -913,7 +913,7 @@ k_fused_tma(const __grid_constant__ CUtensorMap map14, const __grid_constant__ C
         auto load = [&]() {
             const int s = kl % kStages;
             if (lane == 0) {
-                if (!kRead && P.test_stall && kl == 0) {
+                if (P.test_stall == (kRead ? 2 : 1) && kl == 0) {
                     // timeout-path test: the first stage's data never comes; the copy warp waits
                     // (bounded) on a barrier nothing completes, then releases the stage empty
                     if (!mbar_wait(&stall_bar, 0u)) {
@@ -1173,7 +1173,9 @@ k_fused_tma(const __grid_constant__ CUtensorMap map14, const __grid_constant__ C
             block_partial<kComp>((double)r_sum - (double)r_c, (double)t_sum - (double)t_c, partial, item, ct,
                                  kBarComp, red_a, red_b);
         }
-        if (bad) atomicOr(flag, 1);
+        // (a read-out that gave up has formed psi of stages that were never filled; a step that gave up is
+        // reported as such before any non-finite value)
+        if (bad && !(kRead && abort_flag)) atomicOr(flag, 1);
         if constexpr (!kRead) finish_sums<kComp>(partial, n_items, counter, sums_next, ct, kBarComp, red_a, red_b, &is_last);
     } else {
         // ------------------------------------------------------------ halo psi (two warps)
@@ -1228,7 +1230,7 @@ k_fused_tma(const __grid_constant__ CUtensorMap map14, const __grid_constant__ C
                 nb_sync(bar_ring(s), Sh::kCntRing);   // the window is read; the ring holds plane p
             }
         }
-        if (bad) atomicOr(flag, 1);
+        if (bad && !(kRead && abort_flag)) atomicOr(flag, 1);
     }
     __syncthreads();
 }
@@ -1534,7 +1536,9 @@ static int zchunk_readout(const DevParams& P, long long tiles) {
 }
 
 cudaError_t launch_readout(const DevParams& P, int precision, const StateBufs& B, const double* sums_cur, float* rho,
-                           float* ux, float* uy, float* uz, float* T, cudaStream_t s, const TmaMaps* maps) {
+                           float* ux, float* uy, float* uz, float* T, cudaStream_t s, const TmaMaps* maps,
+                           bool* bounded_waits) {
+    *bounded_waits = false;
     // The TMA kernel's read-out instantiation (maps of kReadShape) where its copies pay: from 2^17 nodes
     // (32^3 24 us a call against k_readout's 22, 64 x 64 x 96 33 against 39, 200 x 200 x 300 369 against 527), and
     // not for a frozen g, whose planes z - 1 and z + 1 it would fetch for nothing (181 against 174).
@@ -1545,6 +1549,7 @@ cudaError_t launch_readout(const DevParams& P, int precision, const StateBufs& B
         double* sums_next = nullptr;
         const ReadFields fields{rho, ux, uy, uz, T};
         cudaError_t e = cudaSuccess;
+        *bounded_waits = true;
         if (precision == 0 && P.wet) GB300_TMA(TXR, TYR, float, true, false, true)
         else if (precision == 0) GB300_TMA(TXR, TYR, float, false, false, true)
         else if (precision == 1) GB300_TMA(TXR, TYR, __nv_bfloat16, false, false, true)

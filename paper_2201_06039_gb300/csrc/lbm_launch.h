@@ -111,9 +111,11 @@ int tma_tile_h(int shape);
 
 // macroscopic fields of the current state (B.src) into the device arrays given (each nullable); a
 // scheme-1 wetting wall's table must be that of this state.  With maps (of tile shape tma_read_shape())
-// and a state the TMA kernel reads, its read-out instantiation runs, else k_readout.
+// and a state the TMA kernel reads, its read-out instantiation runs, else k_readout.  *bounded_waits:
+// the launch has waits that can give up (bit 2 of B.flag), after which the fields are not valid.
 cudaError_t launch_readout(const DevParams& P, int precision, const StateBufs& B, const double* sums_cur, float* rho,
-                           float* ux, float* uy, float* uz, float* T, cudaStream_t s, const TmaMaps* maps);
+                           float* ux, float* uy, float* uz, float* T, cudaStream_t s, const TmaMaps* maps,
+                           bool* bounded_waits);
 int tma_read_shape();
 
 // deterministic FP64 sum of a float field into out[0] (out[1] = 0).
