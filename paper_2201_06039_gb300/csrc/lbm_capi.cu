@@ -339,13 +339,15 @@ int enqueue_step(lbm_ctx* c, KernelTimer* timer = nullptr) {
         if (timer) timer->end(0, c->launch);
     } else {
         if (timer) timer->begin(c->launch);
-        // (with u of every node for the finite-difference div u of the collide pass)
-        e = B.vel ? launch_psi_velocity(c->dp, c->p.precision, B, c->sums(c->slot), c->sums(c->slot ^ 1), c->launch)
-                  : launch_psi(c->dp, c->p.precision, B, c->sums(c->slot ^ 1), c->launch);
+        e = launch_psi(c->dp, c->p.precision, B, c->sums(c->slot ^ 1), c->launch);
         if (e != cudaSuccess) return fail(LBM_ECUDA, "psi kernel launch: %s", cudaGetErrorString(e));
         if (timer) {
             timer->end(0, c->launch);
             timer->begin(c->launch);
+        }
+        if (B.vel) {   // u of every node for the finite-difference div u of the collide pass
+            e = launch_velocity(c->dp, c->p.precision, B, c->sums(c->slot), c->launch);
+            if (e != cudaSuccess) return fail(LBM_ECUDA, "velocity kernel launch: %s", cudaGetErrorString(e));
         }
         e = launch_collide(c->dp, c->p.precision, B, c->sums(c->slot), c->first ? 1 : 0, c->launch);
         if (e != cudaSuccess) return fail(LBM_ECUDA, "collide kernel launch: %s", cudaGetErrorString(e));

@@ -20,7 +20,7 @@
 //               pull as one shared-memory load at a fixed offset, and collided planes leave
 //               through TMA tensor stores.  Persistent CTAs take (z-chunk, tile) items round
 //               robin.
-// k_readout   : macroscopic fields (and the first pass of a finite-difference div u step).
+// k_readout   : macroscopic fields.
 #include <cuda.h>
 
 #include <algorithm>
@@ -405,15 +405,11 @@ __device__ __forceinline__ void write_fields(const DevParams& P, const ReadField
 // the ring holds the plane above; then u = (sum e f + F/2) / rho with F from the ring stencil.
 // Populations are read once (the ring's from L2) in place of twice by a psi pass and a moments pass.
 // kBatch: block b of the grid is item b of an ensemble's read-out table, its fields at field_off.
-// kVel: the same pass as the first of a two-pass step with finite-difference div u: (psi, rho) and u of
-// every node (u as the collision forms it) and the FP64 sums of rho and T, in place of a psi pass and
-// a velocity pass that each read the populations.
-template <typename S, int QT, bool kBatch, bool kVel>
+template <typename S, int QT, bool kBatch>
 __global__ void __launch_bounds__(FusedShape<kTY, QT>::kThreads, 2)
 k_readout(DevParams P0, const BatchInst* __restrict__ insts, const BatchItem* __restrict__ items,
           const S* __restrict__ src0, int pull_f, int pull_g, const double* __restrict__ sums_cur, int zchunk,
-          ReadFields out, int* flag, float2* __restrict__ psirho, float4* __restrict__ vel, double2* partial,
-          unsigned* counter, double* sums) {
+          ReadFields out, int* flag) {
     using Sh = FusedShape<kTY, QT>;
     __shared__ float2 ring[Sh::kRing * Sh::kRingPlane];
     int x0, y0, z0, z1, inst = 0;
@@ -472,7 +468,6 @@ k_readout(DevParams P0, const BatchInst* __restrict__ insts, const BatchItem* __
         o.jz = (f[5] - f[6]) + (f[11] - f[12]) - (f[13] - f[14]) + (f[15] - f[16]) - (f[17] - f[18]);
     };
     Node cur = {}, above = {};
-    float ra = 0.f, rc = 0.f, ta = 0.f, tc = 0.f;
     psi_pass(z0 - 1, above);
     psi_pass(z0, cur);
     for (int z = z0; z < z1; ++z) {
@@ -482,34 +477,12 @@ k_readout(DevParams P0, const BatchInst* __restrict__ insts, const BatchItem* __
             const RingStencil rs = ring_stencil(ring + ((z + 3) % Sh::kRing) * Sh::kRingPlane, ring + (z % Sh::kRing) * Sh::kRingPlane,
                                                 ring + ((z + 1) % Sh::kRing) * Sh::kRingPlane,
                                                 bbase(P, slot, -(Sh::kRingW + 1), Sh::kRingW + 1, Sh::kRingPlane), Sh::kRingW);
-            if constexpr (kVel) {
-                const float db = cur.rho - rho_ave;
-                const int d = (int)bidx(P, node_of(P, gx, gy, z), P.N);
-                const Forces F = total_force(P, cur.psi, rs.Fx, rs.Fy, rs.Fz, db);
-                const float inv_rho = __fdividef(1.f, cur.rho);
-                psirho[d] = make_float2(cur.psi, cur.rho);
-                vel[d] = make_float4((cur.jx + 0.5f * F.Fx) * inv_rho, (cur.jy + 0.5f * F.Fy) * inv_rho,
-                                     (cur.jz + 0.5f * F.Fz) * inv_rho, 0.f);
-                kahan_add(ra, rc, cur.rho);
-                kahan_add(ta, tc, cur.T);
-                cur = above;
-                continue;
-            }
             write_fields(P, out, field_off + bidx(P, node_of(P, gx, gy, z), P.N), cur.rho, cur.T, cur.psi, cur.jx, cur.jy,
                          cur.jz, rs, rho_ave);
         }
         cur = above;
     }
     if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(flag, 1);
-    if constexpr (kVel) {
-        __shared__ double red_a[Sh::kThreads / 32], red_b[Sh::kThreads / 32];
-        __shared__ int is_last;
-        const int bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
-        block_partial<Sh::kThreads>((double)ra - (double)rc, (double)ta - (double)tc, partial, bid, threadIdx.x, 0, red_a,
-                                    red_b);
-        finish_sums<Sh::kThreads>(partial, gridDim.x * gridDim.y * gridDim.z, counter, sums, threadIdx.x, 0, red_a, red_b,
-                                  &is_last);
-    }
 }
 
 // ================================================================ TMA kernel
@@ -1560,9 +1533,8 @@ cudaError_t launch_readout(const DevParams& P, int precision, const StateBufs& B
     const int zc = zchunk_readout(P, (long long)tiles_x * tiles_y);
     const dim3 grid(tiles_x, tiles_y, (P.nz + zc - 1) / zc);
 #define GB300_READ(S, QT)                                                                                      \
-    k_readout<S, QT, false, false><<<grid, FusedShape<kTY, QT>::kThreads, 0, s>>>(                             \
-        P, nullptr, nullptr, (const S*)B.src, B.pull_f, B.pull_g, sums_cur, zc, ReadFields{rho, ux, uy, uz, T}, B.flag,    \
-        nullptr, nullptr, nullptr, nullptr, nullptr)
+    k_readout<S, QT, false><<<grid, FusedShape<kTY, QT>::kThreads, 0, s>>>(                                    \
+        P, nullptr, nullptr, (const S*)B.src, B.pull_f, B.pull_g, sums_cur, zc, ReadFields{rho, ux, uy, uz, T}, B.flag)
     if (P.qt == 19) {
         if (precision != 0) return cudaErrorInvalidValue;
         GB300_READ(float, 19);
@@ -1578,37 +1550,12 @@ cudaError_t launch_readout(const DevParams& P, int precision, const StateBufs& B
     return cudaGetLastError();
 }
 
-cudaError_t launch_psi_velocity(const DevParams& P, int precision, const StateBufs& B, const double* sums_cur,
-                                double* sums, cudaStream_t s) {
-    const int tiles_x = (P.nx + TX - 1) / TX, tiles_y = (P.ny + kTY - 1) / kTY;
-    const int zc = zchunk_readout(P, (long long)tiles_x * tiles_y);
-    const dim3 grid(tiles_x, tiles_y, (P.nz + zc - 1) / zc);
-#define GB300_VEL(S, QT)                                                                                       \
-    k_readout<S, QT, false, true><<<grid, FusedShape<kTY, QT>::kThreads, 0, s>>>(                              \
-        P, nullptr, nullptr, (const S*)B.src, B.pull_f, B.pull_g, sums_cur, zc, ReadFields{}, B.flag,     \
-        B.psirho, B.vel, B.partial, B.counter, sums)
-    if (P.qt == 19) {
-        if (precision != 0) return cudaErrorInvalidValue;
-        GB300_VEL(float, 19);
-    } else {
-        switch (precision) {
-        case 0: GB300_VEL(float, 7); break;
-        case 1: GB300_VEL(__nv_bfloat16, 7); break;
-        case 2: GB300_VEL(__half, 7); break;
-        default: return cudaErrorInvalidValue;
-        }
-    }
-#undef GB300_VEL
-    return cudaGetLastError();
-}
-
 cudaError_t launch_readout_batch(const DevParams& P, int precision, const BatchInst* insts, const BatchItem* items,
                                  int n_items, const StateBufs& B, const double* sums_cur, float* rho, float* ux,
                                  float* uy, float* uz, float* T, cudaStream_t s) {
 #define GB300_READ(S)                                                                                          \
-    k_readout<S, 7, true, false><<<n_items, FusedShape<kTY>::kThreads, 0, s>>>(                                \
-        P, insts, items, (const S*)B.src, B.pull_f, B.pull_g, sums_cur, 0, ReadFields{rho, ux, uy, uz, T}, B.flag, nullptr, \
-        nullptr, nullptr, nullptr, nullptr)
+    k_readout<S, 7, true><<<n_items, FusedShape<kTY>::kThreads, 0, s>>>(                                       \
+        P, insts, items, (const S*)B.src, B.pull_f, B.pull_g, sums_cur, 0, ReadFields{rho, ux, uy, uz, T}, B.flag)
     switch (precision) {
     case 0: GB300_READ(float); break;
     case 1: GB300_READ(__nv_bfloat16); break;

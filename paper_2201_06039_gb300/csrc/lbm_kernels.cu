@@ -146,6 +146,34 @@ __device__ __forceinline__ Stencil stencil(const DevParams& P, const float2* __r
     return s;
 }
 
+// ---------------------------------------------------------------- velocity pass
+// u = (sum e f + F/2) / rho (Eq. 10, total force F) of every node, for the finite-difference
+// div u of the collide pass (divu_mode 1); same arithmetic as the collision's u.  A pass of its own: psi,
+// u and the sums in one marching pass read the populations once less, but two planes in (planes a block)
+// more, one after the other, and a step was slower at nearly every size (FP32 pool: 32^3 16.5 against
+// 14.2 us, 64 x 64 x 96 52.8 against 50.7, 96^3 112 against 103, 128^3 253 against 256; BF16 96^3 106
+// against 94; D3Q19 temperature 128^3 391 against 360).
+template <typename S>
+__global__ void __launch_bounds__(TPB) k_velocity(DevParams P, const S* __restrict__ fs, int pull_f,
+                                                 const float2* __restrict__ psirho,
+                                                 const double* __restrict__ sums_cur, float4* __restrict__ vel) {
+    int x = blockIdx.x * TPB_X + threadIdx.x, y = blockIdx.y * TPB_Y + threadIdx.y, z = blockIdx.z;
+    if (x >= P.nx || y >= P.ny) return;
+    int i = sidx(P, x, y, z), d = (int)bidx(P, node_of(P, x, y, z), P.N);
+    Nbr n = make_nbr(P, x, y, z);
+    float f[19];
+    load_f<S>(P, fs, pull_f, i, x, y, z, n, f);
+    float rho = sum19(f);
+    float jx = (f[1] - f[2]) + (f[7] - f[8]) + (f[9] - f[10]) + (f[11] - f[12]) + (f[13] - f[14]);
+    float jy = (f[3] - f[4]) + (f[7] - f[8]) - (f[9] - f[10]) + (f[15] - f[16]) + (f[17] - f[18]);
+    float jz = (f[5] - f[6]) + (f[11] - f[12]) - (f[13] - f[14]) + (f[15] - f[16]) - (f[17] - f[18]);
+    float2 me = __ldg(psirho + d);
+    Stencil st = stencil(P, psirho, x, y, z, n);
+    const Forces F = total_force(P, me.x, st.x.x, st.y.x, st.z.x, rho - buoyancy_ref(P, sums_cur[0], P.inv_N));
+    const float inv_rho = __fdividef(1.f, rho);
+    vel[d] = make_float4((jx + 0.5f * F.Fx) * inv_rho, (jy + 0.5f * F.Fy) * inv_rho, (jz + 0.5f * F.Fz) * inv_rho, 0.f);
+}
+
 // Does the gradient stencil of (x, y, z) reach past a wall or outflow face?  There div u stays
 // Eq. 48 in divu_mode 1.
 __device__ __forceinline__ bool next_to_solid(const DevParams& P, int x, int y, int z) {
@@ -355,6 +383,14 @@ cudaError_t launch_wall_table(const DevParams& P, int precision, const void* fs,
                               cudaStream_t s) {
     const dim3 grid((P.nx + TPB_X - 1) / TPB_X, (P.ny + TPB_Y - 1) / TPB_Y), blk(TPB_X, TPB_Y);
     GB300_DISPATCH(precision, (k_wall_table<S><<<grid, blk, 0, s>>>(P, (const S*)fs, pull_f, tab)));
+    return cudaGetLastError();
+}
+
+cudaError_t launch_velocity(const DevParams& P, int precision, const StateBufs& B, const double* sums_cur,
+                            cudaStream_t s) {
+    dim3 blk(TPB_X, TPB_Y);
+    GB300_DISPATCH(precision, (k_velocity<S><<<grid_of(P), blk, 0, s>>>(P, (const S*)B.src, B.pull_f, B.psirho,
+                                                                         sums_cur, B.vel)));
     return cudaGetLastError();
 }
 

@@ -31,9 +31,9 @@ cudaError_t launch_init(const DevParams& P, int precision, void* pops, const flo
 cudaError_t launch_psi(const DevParams& P, int precision, const StateBufs& B, double* sums,
                        cudaStream_t s);
 
-// the psi pass with u = (sum e f + F/2) / rho of every node into B.vel (finite-difference div u)
-cudaError_t launch_psi_velocity(const DevParams& P, int precision, const StateBufs& B, const double* sums_cur,
-                                double* sums, cudaStream_t s);
+// u = (sum e f + F/2) / rho of every node into B.vel (finite-difference div u)
+cudaError_t launch_velocity(const DevParams& P, int precision, const StateBufs& B, const double* sums_cur,
+                            cudaStream_t s);
 cudaError_t launch_wall_params(const DevParams& P, float2* par, cudaStream_t s);
 cudaError_t launch_wall_map(const DevParams& P, const float* phi, const float* drho, float2* par, int* bad,
                             int write, cudaStream_t s);
