@@ -266,7 +266,8 @@ int enqueue_tma_steps(lbm_batch* b, int m) {
         const TmaMaps* maps = &b->tmaps[k];
         StateBufs B0 = b->bufs(k);
         // a state the batched kernel wrote: refresh its ghost cells before the first TMA launch
-        if (!fresh0 && !b->ghosts_valid && maps->ok) e = launch_ghosts(b->dps[k], b->p.precision, (void*)B0.src, s);
+        const bool ghosts = maps->ok && maps->ghosts != 3;   // 3: no pull reads a ghost cell
+        if (!fresh0 && !b->ghosts_valid && ghosts) e = launch_ghosts(b->dps[k], b->p.precision, (void*)B0.src, s);
         for (int j = 0; j < m && e == cudaSuccess; ++j) {
             const int cur = b->cur ^ (j & 1), slot = b->slot ^ (j & 1);
             // a frozen field (flow_off / thermal_off) keeps its un-streamed form on every step
@@ -284,7 +285,7 @@ int enqueue_tma_steps(lbm_batch* b, int m) {
             e = launch_fused(b->dps[k], b->p.precision, B, b->sums(slot) + 2 * k, b->sums(slot ^ 1) + 2 * k,
                              j == 0 && b->first ? 1 : 0, s, maps, &ghosts_done);
             // the next TMA launch reads ghost cells (the generic kernel wraps its pulls itself)
-            if (e == cudaSuccess && !ghosts_done && maps->ok) e = launch_ghosts(b->dps[k], b->p.precision, B.dst, s);
+            if (e == cudaSuccess && !ghosts_done && ghosts) e = launch_ghosts(b->dps[k], b->p.precision, B.dst, s);
         }
     }
     for (int q = 0; q < kSide && e == cudaSuccess; ++q) {

@@ -318,6 +318,11 @@ struct KernelTimer {
     }
 };
 
+// Will the context's next launch read the ghost cells of the current buffer?  Only the TMA kernel does, on
+// lattices whose pulls wrap across x or y and once the state is in the form it reads: not right after
+// lbm_init_fields, and not with a frozen g in streamed form, which stays with the generic kernel.
+bool reads_ghosts(lbm_ctx* c) { return c->maps.ok && c->maps.ghosts != 3 && tma_runs(c->dp, c->p.precision, c->bufs()); }
+
 // Enqueue one time step of the selected variant on the context's stream (each launch timed when
 // a timer is given).
 int enqueue_step(lbm_ctx* c, KernelTimer* timer = nullptr) {
@@ -356,14 +361,14 @@ int enqueue_step(lbm_ctx* c, KernelTimer* timer = nullptr) {
     // both fields are written every step (frozen ones copied through unchanged, so they stay
     // in their un-streamed "fresh" form)
     c->cur ^= 1;
-    if (c->maps.ok && !ghosts_done) {   // the TMA path reads ghost cells: refresh them in the state just written
+    if (!c->p.flow_off) c->fresh_f = false;
+    if (!c->p.thermal_off) c->fresh_g = false;
+    if (!ghosts_done && reads_ghosts(c)) {   // refresh the ghost cells of the state just written
         if (timer) timer->begin(c->launch);
         e = launch_ghosts(c->dp, c->p.precision, B.dst, c->launch);
         if (e != cudaSuccess) return fail(LBM_ECUDA, "ghost refresh launch: %s", cudaGetErrorString(e));
         if (timer) timer->end(2, c->launch);
     }
-    if (!c->p.flow_off) c->fresh_f = false;
-    if (!c->p.thermal_off) c->fresh_g = false;
     c->slot ^= 1;
     c->first = false;
     c->steps += 1;
@@ -685,7 +690,6 @@ int lbm_init_fields(lbm_ctx* c, const float* rho, const float* T, const float* u
     c->cur = 0;
     c->slot = 0;
     CK(launch_init(c->dp, c->p.precision, c->pbuf(0), drho, dT, du, c->stream));
-    if (c->maps.ok) CK(launch_ghosts(c->dp, c->p.precision, c->pbuf(0), c->stream));
     StateBufs B = c->bufs();
     CK(launch_sum_field(drho, c->dp.N, B.partial, B.counter, c->sums(0), c->stream));
     CK(cudaMemsetAsync(c->base + c->L.flag, 0, sizeof(int), c->stream));
@@ -870,12 +874,12 @@ int lbm_load_state(lbm_ctx* c, const void* buf, size_t bytes) {
     CK(cudaMemcpyAsync(c->base + c->L.phis, in + h.pop_bytes, (size_t)h.phis_bytes, cudaMemcpyHostToDevice, c->stream));
     CK(cudaMemcpyAsync(c->sums(c->slot), in + h.pop_bytes + h.phis_bytes, 2 * sizeof(double), cudaMemcpyHostToDevice,
                        c->stream));
-    // the saving context may not have kept the ghost cells (kernels without TMA do not use them)
-    if (c->maps.ok && !(h.fresh_f && h.fresh_g)) CK(launch_ghosts(c->dp, c->p.precision, c->pbuf(c->cur), c->stream));
-    CK(cudaMemsetAsync(c->base + c->L.flag, 0, sizeof(int), c->stream));
-    CK(cudaStreamSynchronize(c->stream));
     c->fresh_f = h.fresh_f != 0;
     c->fresh_g = h.fresh_g != 0;
+    // the saving context may not have kept the ghost cells (kernels without TMA do not use them)
+    if (reads_ghosts(c)) CK(launch_ghosts(c->dp, c->p.precision, c->pbuf(c->cur), c->stream));
+    CK(cudaMemsetAsync(c->base + c->L.flag, 0, sizeof(int), c->stream));
+    CK(cudaStreamSynchronize(c->stream));
     c->first = h.first != 0;
     c->steps = h.steps;
     c->initialised = true;
