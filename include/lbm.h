@@ -210,7 +210,8 @@ int lbm_set_wall_map(lbm_ctx* ctx, const float* phi, const float* drho);
 
 /* Kernel variant the context runs (LBM_KERNEL_TWO_PASS, LBM_KERNEL_FUSED or
  * LBM_KERNEL_FUSED_TMA; AUTO resolved).  The first step after lbm_init_fields always runs the
- * generic fused kernel. */
+ * generic fused kernel, and so does every step of a frozen-temperature context on a loaded checkpoint
+ * of a run with temperature (LBM_KERNEL_FUSED until the next lbm_init_fields). */
 int lbm_kernel_in_use(const lbm_ctx* ctx);
 
 /* Tile plan of the TMA kernel (the default path; see LBM_KERNEL_FUSED_TMA for what it covers).  A

@@ -323,6 +323,12 @@ struct KernelTimer {
 // lbm_init_fields, and not with a frozen g in streamed form, which stays with the generic kernel.
 bool reads_ghosts(lbm_ctx* c) { return c->maps.ok && c->maps.ghosts != 3 && tma_runs(c->dp, c->p.precision, c->bufs()); }
 
+// Do the context's steps run on the TMA kernel (the first one after lbm_init_fields aside)?  With a frozen g
+// loaded in streamed form they stay with the generic kernel until the next lbm_init_fields.
+bool steps_on_tma(const lbm_ctx* c) {
+    return c->variant == LBM_KERNEL_FUSED && c->maps.ok && !(c->p.thermal_off && c->initialised && !c->fresh_g);
+}
+
 // Enqueue one time step of the selected variant on the context's stream (each launch timed when
 // a timer is given).
 int enqueue_step(lbm_ctx* c, KernelTimer* timer = nullptr) {
@@ -897,7 +903,7 @@ int lbm_plan_shapes(int* tile_w, int* tile_h, int max) {
 
 int lbm_get_plan(const lbm_ctx* c, int* shape, int* zchunk, int* items, int* ctas) {
     if (!c) return fail(LBM_EINVAL, "ctx is NULL");
-    const bool ok = c->maps.ok;
+    const bool ok = steps_on_tma(c);
     if (shape) *shape = ok ? c->maps.shape : -1;
     if (zchunk) *zchunk = ok ? c->maps.zchunk : 0;
     if (items) *items = ok ? c->maps.items : 0;
@@ -930,8 +936,7 @@ int lbm_autotune(lbm_ctx* c, int steps, double* best_ms) {
     if (!c) return fail(LBM_EINVAL, "ctx is NULL");
     if (!c->initialised) return fail(LBM_ESTATE, "lbm_autotune before lbm_init_fields");
     if (steps < 1) return fail(LBM_EINVAL, "steps must be >= 1");
-    if (c->variant != LBM_KERNEL_FUSED || c->p.use_tma == 0 || !c->maps.ok)
-        return fail(LBM_ESTATE, "the context does not run the TMA kernel");
+    if (!steps_on_tma(c)) return fail(LBM_ESTATE, "the context does not run the TMA kernel");
     // the first step after lbm_init_fields runs the generic kernel: take it before timing
     int rc = LBM_OK;
     while (rc == LBM_OK && (c->first || (c->fresh_f && !c->p.flow_off) || (c->fresh_g && !c->p.thermal_off))) rc = enqueue_step(c);
@@ -1015,8 +1020,7 @@ int lbm_autotune(lbm_ctx* c, int steps, double* best_ms) {
 
 int lbm_kernel_in_use(const lbm_ctx* c) {
     if (!c) return LBM_EINVAL;
-    if (c->variant == LBM_KERNEL_FUSED && c->maps.ok) return LBM_KERNEL_FUSED_TMA;
-    return c->variant;
+    return steps_on_tma(c) ? LBM_KERNEL_FUSED_TMA : c->variant;
 }
 
 void lbm_destroy(lbm_ctx* c) {
