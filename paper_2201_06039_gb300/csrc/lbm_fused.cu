@@ -1286,6 +1286,14 @@ double tma_cost(int shape, long long items, int zc, int ctas) {
     return (double)((items + ctas - 1) / ctas) * kTmaTX[shape] * kTmaTY[shape] / kTmaRate[shape] * (zc + 2.1);
 }
 
+// The next smaller z-chunk after zc among ceil(nz / n), n = 1, 2, ..., or 0 after one plane: about 2 sqrt(nz)
+// of them.  (Counted through every n, the plans of a 16 x 16 x 8000 lattice took 0.35 ms of lbm_create.)
+int next_zchunk(int nz, int zc) {
+    if (zc <= 1) return 0;
+    const int n = (nz + zc - 2) / (zc - 1);   // the smallest n with ceil(nz / n) < zc
+    return (nz + n - 1) / n;
+}
+
 // Plan of the TMA kernel for a lattice: the tile shape and z-chunking of least modelled time among
 // those of at most max_items items.  forced_shape / forced_zchunk (>= 0 / > 0) pin either choice.
 // lbm_autotune replaces the model by measurement.
@@ -1297,9 +1305,8 @@ void tma_plan(const DevParams& P, int ctas, int forced_shape, int forced_zchunk,
         if (forced_shape >= 0 && sh != forced_shape) continue;
         const int tx = kTmaTX[sh], ty = kTmaTY[sh];
         const int tiles = ((P.nx + tx - 1) / tx) * ((P.ny + ty - 1) / ty);
-        for (int nch = 1; nch <= P.nz; ++nch) {
-            int zc = (P.nz + nch - 1) / nch;
-            if (forced_zchunk > 0) zc = forced_zchunk < P.nz ? forced_zchunk : P.nz;
+        for (int zc = forced_zchunk > 0 ? (forced_zchunk < P.nz ? forced_zchunk : P.nz) : P.nz; zc > 0;
+             zc = forced_zchunk > 0 ? 0 : next_zchunk(P.nz, zc)) {
             const long long n = (long long)tiles * ((P.nz + zc - 1) / zc);
             const double cost = tma_cost(sh, n, zc, ctas);
             if (n <= max_items && (best < 0 || cost < best)) {
@@ -1308,7 +1315,6 @@ void tma_plan(const DevParams& P, int ctas, int forced_shape, int forced_zchunk,
                 *zchunk = zc;
                 *items = (int)n;
             }
-            if (forced_zchunk > 0) break;
         }
     }
 }
@@ -1387,9 +1393,7 @@ int tma_zchunk_candidates(const DevParams& P, int ctas, int shape, int* zcs, int
     int n = 0;
     double cost[64];
     int zc_of[64];
-    for (int nch = 1; nch <= P.nz && n < 64; ++nch) {
-        const int zc = (P.nz + nch - 1) / nch;
-        if (n > 0 && zc_of[n - 1] == zc) continue;
+    for (int zc = P.nz; zc > 0 && n < 64; zc = next_zchunk(P.nz, zc)) {
         cost[n] = tma_cost(shape, tiles * ((P.nz + zc - 1) / zc), zc, ctas);
         zc_of[n++] = zc;
     }
