@@ -151,15 +151,25 @@ int items_of_plan(const lbm_batch* b, const Plan& pl, std::vector<BatchItem>* it
     return count;
 }
 
-// Items of the one-launch read-out: 32 x 8 tiles and chunks of 16 planes (two of the 18 planes a block
-// reads are read by the next block too), instances largest first.
+// Items of the one-launch read-out: 32 x 8 tiles and chunks of planes (two planes more are read than
+// written), instances largest first.  The chunks are as short as two blocks an SM allow, at most 16
+// planes: a small ensemble would leave the GPU idle on long ones (one 32^3 47 us a call with 16 planes, 28
+// with one; two of 64 x 64 x 70 51, 46 with eight), a large one would read its two planes too often (64 of
+// 33 x 31 x 35 200 us with 16 planes, 234 with four).
 void readout_items(const lbm_batch* b, std::vector<BatchItem>* items) {
+    auto count = [&](int zc) {
+        long long n = 0;
+        for (const DevParams& d : b->dps) n += (long long)((d.nx + 31) / 32) * ((d.ny + 7) / 8) * ((d.nz + zc - 1) / zc);
+        return n;
+    };
+    int zc = 1;
+    while (zc < 16 && count(zc) > 2 * b->sms) ++zc;
     for (int idx = 0; idx < b->n; ++idx) {
         const int k = b->order[idx];
         const DevParams& d = b->dps[k];
-        for (int z = 0; z < d.nz; z += 16)
+        for (int z = 0; z < d.nz; z += zc)
             for (int y = 0; y < d.ny; y += 8)
-                for (int x = 0; x < d.nx; x += 32) items->push_back(BatchItem{k, x, y, z, std::min(d.nz, z + 16), 0});
+                for (int x = 0; x < d.nx; x += 32) items->push_back(BatchItem{k, x, y, z, std::min(d.nz, z + zc), 0});
     }
 }
 
@@ -482,6 +492,12 @@ int lbm_batch_create(const lbm_params* common, int n_instances, const int* dims,
     }
     if (t_total < (1LL << 30)) b->max_partial = std::max(b->max_partial, (int)t_total);
 
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        cudaGetLastError();
+        delete b;
+        return fail(LBM_ECUDA, "no CUDA device");
+    }
     const size_t pb = pop_bytes(common->precision);
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off = align256(off + bytes); return o; };
@@ -505,12 +521,6 @@ int lbm_batch_create(const lbm_params* common, int n_instances, const int* dims,
     b->ghosts_valid = false;
     b->t_items = 0;
     b->t_launches = 0;
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-        cudaGetLastError();
-        delete b;
-        return fail(LBM_ECUDA, "no CUDA device");
-    }
     cudaError_t e = cudaMalloc((void**)&b->base, off);
     if (e != cudaSuccess) {
         cudaGetLastError();
