@@ -30,6 +30,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <functional>
 #include <numeric>
 #include <vector>
 
@@ -178,11 +179,43 @@ void drop_batch_graphs(lbm_batch* b) {
     b->n_graphs = 0;
 }
 
+// Modelled time of a step whose launches (microseconds each) go to the side streams, longest first, each to
+// the stream with the least so far.
+double busiest_stream(std::vector<double> t) {
+    std::sort(t.begin(), t.end(), std::greater<double>());
+    std::vector<double> load(kSide, 0.0);
+    for (double v : t) *std::min_element(load.begin(), load.end()) += v;
+    return *std::max_element(load.begin(), load.end());
+}
+
+// Does the TMA mode pay on instances with walls or outflow across x or y or with a frozen temperature, over
+// the generic kernel in its place?  A launch lasts about 11 us and 2.3 a plane of its longest item: whole or
+// half columns here, chunks of 8 planes or more there, which small instances are done with sooner.  The
+// generic kernel's rate, 12500 nodes a microsecond in 32 x 8 tiles, and the columns' share of the SMs bound
+// the two for many.  Measured, TMA against generic, us a step: closed boxes 1 x 32^3 89 / 33, 64 x 32^3
+// 211 / 182, 2 x (64 x 64 x 70) 99 / 54, 4 x 101 / 89, 5 x 104 / 111, 8 x 127 / 175, 3 x 96^3 153 / 192, 16 x
+// (20 x 20 x 100) 139 / 94, 32 x 154 / 184; frozen 1 x 32^3 96 / 30, 8 x (64 x 64 x 70) 157 / 156, 3 x 96^3 159 / 174.
+bool columns_pay(const lbm_batch* b) {
+    std::vector<double> col(b->n), gen(b->n);
+    double col_work = 0.0, gen_nodes = 0.0;
+    for (int k = 0; k < b->n; ++k) {
+        const DevParams& d = b->dps[k];
+        const TmaMaps& m = b->tmaps[k];
+        gen[k] = 11.0 + 2.3 * (std::min(d.nz, 8) + 2);
+        col[k] = m.ok ? 11.0 + 2.3 * (m.zchunk + 2) : gen[k];
+        col_work += m.ok ? col[k] * m.items : 0.0;
+        gen_nodes += (double)((d.nx + 31) / 32 * 32) * ((d.ny + 7) / 8 * 8) * d.nz;
+    }
+    return std::max(busiest_stream(col), col_work / b->sms) < std::max(busiest_stream(gen), gen_nodes / 12500.0);
+}
+
 // TMA mode: tensor maps and plan of every instance: whole- or half-column items and the tile shape with
 // the least padded volume per node rate (the plan model for one CTA: the instances share the
 // GPU; on the 256-instance ensemble 15.2k MLUPS against 14.4k for the model's single-lattice
 // choice, the smallest tile); then the instances go to the side streams longest first, each to
 // the stream with the least modelled work so far, so that the streams reach each join together.
+// Ensembles with walls or outflow across x or y or with a frozen temperature run the generic kernel here
+// where that is faster (columns_pay).
 // LBM_ESTATE if an instance runs neither the TMA nor the generic fused kernel.
 int set_tma_plan(lbm_batch* b) {
     if (!b->side_ok) {
@@ -212,8 +245,14 @@ int set_tma_plan(lbm_batch* b) {
                         d.nx, d.ny, d.nz);
         b->t_part[k] = off;
         off += b->t_cap[k];
-        launches += tma && !b->tmaps[k].ghosts ? 2 : 1;
-        ctas += tma ? std::min(b->tmaps[k].items, b->tmaps[k].sms) : (int)fused_blocks(d);
+    }
+    const DevParams& d0 = b->dps[0];   // faces and frozen fields are the ensemble's
+    if (((d0.xy_walls | d0.xy_open) != 0 || d0.thermal_off) && !columns_pay(b))
+        for (TmaMaps& m : b->tmaps) m.ok = false;
+    for (int k = 0; k < b->n; ++k) {
+        const TmaMaps& m = b->tmaps[k];
+        launches += m.ok && !m.ghosts ? 2 : 1;
+        ctas += m.ok ? std::min(m.items, m.sms) : (int)fused_blocks(b->dps[k]);
     }
     b->t_items = off;
     b->t_launches = launches;
