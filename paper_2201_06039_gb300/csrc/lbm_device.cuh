@@ -411,6 +411,27 @@ __device__ __forceinline__ void back_transform(float rho, float ax, float bx, fl
     f[0] = rho - s;
 }
 
+// ---------------------------------------------------------------- read-out
+struct ReadFields {   // device arrays, each nullable
+    float *rho, *ux, *uy, *uz, *T;
+};
+// the fields of one node (dense index d): u = (j + F/2) / rho, F = F_m + (rho - rho_ave) g from the stencil
+// sums (sx, sy, sz)
+__device__ __forceinline__ void write_fields(const DevParams& P, const ReadFields& out, long long d, float rho, float T,
+                                             float psi, float jx, float jy, float jz, float sx, float sy, float sz,
+                                             float rho_ave) {
+    const float db = rho - rho_ave;
+    const float Fx = __fmaf_rn(psi, sx, __fmul_rn(db, P.gx)), Fy = __fmaf_rn(psi, sy, __fmul_rn(db, P.gy)),
+                Fz = __fmaf_rn(psi, sz, __fmul_rn(db, P.gz));
+    const float inv = 1.f / rho;
+    const bool fz = P.flow_off != 0;
+    if (out.rho) out.rho[d] = rho;
+    if (out.ux) out.ux[d] = fz ? 0.f : (jx + 0.5f * Fx) * inv;
+    if (out.uy) out.uy[d] = fz ? 0.f : (jy + 0.5f * Fy) * inv;
+    if (out.uz) out.uz[d] = fz ? 0.f : (jz + 0.5f * Fz) * inv;
+    if (out.T) out.T[d] = T;
+}
+
 // ---------------------------------------------------------------- D3Q19 MRT collision
 // One moment of Eq. 3: m* = m - L (m - m_eq) + (1 - L/2) S = m + (-L (m - m_eq) + h S), with every
 // rounding step explicit.  Written as plain arithmetic the sum of two products leaves the compiler

@@ -381,24 +381,6 @@ k_fused_batch(DevParams P, const BatchInst* __restrict__ insts, const BatchItem*
 }
 
 // ================================================================ read-out
-struct ReadFields {   // device arrays, each nullable
-    float *rho, *ux, *uy, *uz, *T;
-};
-// the fields of one node: u = (j + F/2) / rho, F = F_m + (rho - rho_ave) g
-__device__ __forceinline__ void write_fields(const DevParams& P, const ReadFields& out, long long d, float rho, float T,
-                                             float psi, float jx, float jy, float jz, const RingStencil& rs, float rho_ave) {
-    const float db = rho - rho_ave;
-    const float Fx = __fmaf_rn(psi, rs.Fx, __fmul_rn(db, P.gx)), Fy = __fmaf_rn(psi, rs.Fy, __fmul_rn(db, P.gy)),
-                Fz = __fmaf_rn(psi, rs.Fz, __fmul_rn(db, P.gz));
-    const float inv = 1.f / rho;
-    const bool fz = P.flow_off != 0;
-    if (out.rho) out.rho[d] = rho;
-    if (out.ux) out.ux[d] = fz ? 0.f : (jx + 0.5f * Fx) * inv;
-    if (out.uy) out.uy[d] = fz ? 0.f : (jy + 0.5f * Fy) * inv;
-    if (out.uz) out.uz[d] = fz ? 0.f : (jz + 0.5f * Fz) * inv;
-    if (out.T) out.T[d] = T;
-}
-
 // Macroscopic fields in one pass over the populations: a block marches a 32 x 8 tile through a chunk
 // of planes; every thread pulls its node (or a node of the ring around the tile), puts (psi, rho) into
 // a four-plane shared ring and keeps rho, T and the first moment of its node for one plane, until
@@ -478,7 +460,7 @@ k_readout(DevParams P0, const BatchInst* __restrict__ insts, const BatchItem* __
                                                 ring + ((z + 1) % Sh::kRing) * Sh::kRingPlane,
                                                 bbase(P, slot, -(Sh::kRingW + 1), Sh::kRingW + 1, Sh::kRingPlane), Sh::kRingW);
             write_fields(P, out, field_off + bidx(P, node_of(P, gx, gy, z), P.N), cur.rho, cur.T, cur.psi, cur.jx, cur.jy,
-                         cur.jz, rs, rho_ave);
+                         cur.jz, rs.Fx, rs.Fy, rs.Fz, rho_ave);
         }
         cur = above;
     }
@@ -1114,7 +1096,8 @@ k_fused_tma(const __grid_constant__ CUtensorMap map14, const __grid_constant__ C
                     if (owner) {
                         const RingStencil rs = ring_stencil(ring + ((k - 3) % kRing) * kRP, ring + ((k - 2) % kRing) * kRP,
                                                             ring + ((k - 1) % kRing) * kRP, slot, Sh::kRingW);
-                        write_fields(P, out, bidx(P, node_of(P, gx, gy, z), P.N), rho, T, psi, jx, jy, jz, rs, rho_ave);
+                        write_fields(P, out, bidx(P, node_of(P, gx, gy, z), P.N), rho, T, psi, jx, jy, jz, rs.Fx, rs.Fy,
+                                     rs.Fz, rho_ave);
                     }
                     moment();
                     rho = rho_n;
@@ -1516,10 +1499,22 @@ cudaError_t launch_readout(const DevParams& P, int precision, const StateBufs& B
                            float* ux, float* uy, float* uz, float* T, cudaStream_t s, const TmaMaps* maps,
                            bool* bounded_waits) {
     *bounded_waits = false;
+    // Thin lattices of some size: a psi pass and a moments pass.  A block that marches planes reads two more
+    // than it writes, which a few planes do not repay: 512 x 512 x 1 k_readout 44 us a call, two passes 37;
+    // 512 x 512 x 2 54, 47; D3Q19 temperature 87, 77; below 2^16 nodes the second launch costs as much (64 x 64 x 1
+    // 25, 27).
+    if (P.nz <= 3 && P.N >= 1 << 16) {
+        const cudaError_t e = launch_psi(P, precision, B, nullptr, s);
+        return e != cudaSuccess ? e : launch_moments(P, precision, B, sums_cur, ReadFields{rho, ux, uy, uz, T}, s);
+    }
     // The TMA kernel's read-out instantiation (maps of kReadShape) where its copies pay: from 2^17 nodes
     // (32^3 24 us a call against k_readout's 22, 64 x 64 x 96 33 against 39, 200 x 200 x 300 369 against 527), and
-    // not for a frozen g, whose planes z - 1 and z + 1 it would fetch for nothing (181 against 174).
-    if (maps && maps->ok && P.N >= 1 << 17 && !P.thermal_off && tma_runs(P, precision, B)) {
+    // not for a frozen g, whose planes z - 1 and z + 1 it would fetch for nothing (181 against 174).  Walls or
+    // outflow across x or y, whose patches weigh more there, need planes to make up for them (closed boxes
+    // of 512 x 512 x 4 89 against 83, in BF16 87 against 79; of 200 x 200 x 8 42 against 43, 46 against 44; of
+    // 96^3 59 against 69, 62 against 65).
+    const bool faces = (P.xy_walls | P.xy_open) != 0;
+    if (maps && maps->ok && P.N >= 1 << 17 && !(faces && P.nz <= 8) && !P.thermal_off && tma_runs(P, precision, B)) {
         constexpr int TXR = kTmaTX[kReadShape], TYR = kTmaTY[kReadShape];
         const int txs = (P.nx + TXR - 1) / TXR, tys = (P.ny + TYR - 1) / TYR;
         const int ctas = maps->sms < maps->items ? maps->sms : maps->items, first = 0;

@@ -239,6 +239,28 @@ __global__ void __launch_bounds__(TPB, QT == 7 ? 3 : 2) k_collide(DevParams P, c
     phis[d] = ph;
 }
 
+// ---------------------------------------------------------------- moments pass
+// Macroscopic fields of every node from its pulled populations and the (psi, rho) field: the read-out of
+// thin lattices (see launch_readout), bit for bit that of the marching kernels.
+template <typename S, int QT>
+__global__ void __launch_bounds__(TPB) k_moments(DevParams P, const S* __restrict__ fs, int pull_f, int pull_g,
+                                                const float2* __restrict__ psirho, const double* __restrict__ sums_cur,
+                                                ReadFields out) {
+    int x = blockIdx.x * TPB_X + threadIdx.x, y = blockIdx.y * TPB_Y + threadIdx.y, z = blockIdx.z;
+    if (x >= P.nx || y >= P.ny) return;
+    int i = sidx(P, x, y, z), d = (int)bidx(P, node_of(P, x, y, z), P.N);
+    Nbr n = make_nbr(P, x, y, z);
+    float f[19], g[QT];
+    load_f<S>(P, fs, pull_f, i, x, y, z, n, f);
+    Therm<QT>::template load<S>(P, fs, pull_g, i, x, y, z, n, g);
+    float jx = (f[1] - f[2]) + (f[7] - f[8]) + (f[9] - f[10]) + (f[11] - f[12]) + (f[13] - f[14]);
+    float jy = (f[3] - f[4]) + (f[7] - f[8]) - (f[9] - f[10]) + (f[15] - f[16]) + (f[17] - f[18]);
+    float jz = (f[5] - f[6]) + (f[11] - f[12]) - (f[13] - f[14]) + (f[15] - f[16]) - (f[17] - f[18]);
+    Stencil st = stencil(P, psirho, x, y, z, n);
+    write_fields(P, out, d, sum19(f), Therm<QT>::sum(g), __ldg(psirho + d).x, jx, jy, jz, st.x.x, st.y.x, st.z.x,
+                 buoyancy_ref(P, sums_cur[0], P.inv_N));
+}
+
 // ---------------------------------------------------------------- field sum
 __global__ void __launch_bounds__(256) k_sum_field(const float* __restrict__ a, int n, double2* partial,
                                                    unsigned* counter, double* out) {
@@ -290,8 +312,8 @@ cudaError_t launch_init(const DevParams& P, int precision, void* pops, const flo
 
 cudaError_t launch_psi(const DevParams& P, int precision, const StateBufs& B, double* sums, cudaStream_t s) {
     dim3 blk(TPB_X, TPB_Y), grid = grid_of(P);
-    // one round of three blocks an SM, at most 16 planes a block
-    const int zc = (int)std::max(1LL, std::min(16LL, ((long long)grid.x * grid.y * grid.z + 455) / 456));
+    // with sums: one round of three blocks an SM, at most 16 planes a block; without, a plane a block
+    const int zc = !sums ? 1 : (int)std::max(1LL, std::min(16LL, ((long long)grid.x * grid.y * grid.z + 455) / 456));
     grid.z = (P.nz + zc - 1) / zc;
     GB300_DISPATCH_QT(P, precision, (k_psi<S, QT><<<grid, blk, 0, s>>>(P, (const S*)B.src, B.pull_f, B.pull_g, B.psirho,
                                                                        B.partial, B.counter, sums, B.flag, zc)));
@@ -391,6 +413,14 @@ cudaError_t launch_velocity(const DevParams& P, int precision, const StateBufs& 
     dim3 blk(TPB_X, TPB_Y);
     GB300_DISPATCH(precision, (k_velocity<S><<<grid_of(P), blk, 0, s>>>(P, (const S*)B.src, B.pull_f, B.psirho,
                                                                          sums_cur, B.vel)));
+    return cudaGetLastError();
+}
+
+cudaError_t launch_moments(const DevParams& P, int precision, const StateBufs& B, const double* sums_cur,
+                           const ReadFields& out, cudaStream_t s) {
+    dim3 blk(TPB_X, TPB_Y);
+    GB300_DISPATCH_QT(P, precision, (k_moments<S, QT><<<grid_of(P), blk, 0, s>>>(P, (const S*)B.src, B.pull_f, B.pull_g,
+                                                                        B.psirho, sums_cur, out)));
     return cudaGetLastError();
 }
 

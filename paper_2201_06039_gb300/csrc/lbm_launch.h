@@ -34,6 +34,9 @@ cudaError_t launch_psi(const DevParams& P, int precision, const StateBufs& B, do
 // u = (sum e f + F/2) / rho of every node into B.vel (finite-difference div u)
 cudaError_t launch_velocity(const DevParams& P, int precision, const StateBufs& B, const double* sums_cur,
                             cudaStream_t s);
+// macroscopic fields of every node (each array nullable) from the populations and B.psirho of a psi pass
+cudaError_t launch_moments(const DevParams& P, int precision, const StateBufs& B, const double* sums_cur,
+                           const ReadFields& out, cudaStream_t s);
 cudaError_t launch_wall_params(const DevParams& P, float2* par, cudaStream_t s);
 cudaError_t launch_wall_map(const DevParams& P, const float* phi, const float* drho, float2* par, int* bad,
                             int write, cudaStream_t s);
@@ -111,8 +114,9 @@ int tma_tile_h(int shape);
 
 // macroscopic fields of the current state (B.src) into the device arrays given (each nullable); a
 // scheme-1 wetting wall's table must be that of this state.  With maps (of tile shape tma_read_shape())
-// and a state the TMA kernel reads, its read-out instantiation runs, else k_readout.  *bounded_waits:
-// the launch has waits that can give up (bit 2 of B.flag), after which the fields are not valid.
+// and a state the TMA kernel reads, its read-out instantiation runs, else k_readout; on thin lattices a psi
+// pass (into B.psirho) and a moments pass.  *bounded_waits: the launch has waits that can give up (bit 2 of
+// B.flag), after which the fields are not valid.
 cudaError_t launch_readout(const DevParams& P, int precision, const StateBufs& B, const double* sums_cur, float* rho,
                            float* ux, float* uy, float* uz, float* T, cudaStream_t s, const TmaMaps* maps,
                            bool* bounded_waits);
