@@ -172,9 +172,8 @@ int lbm_step(lbm_ctx* ctx, int n);
 /* Macroscopic fields of the current state: rho = sum f (Eq. 10), u = (sum e f + F/2)/rho
  * (Eq. 10, F = F_m of Eq. 7 + F_b with the rho_ave the next step uses), T = sum g (Eq. 20).
  * Any output pointer may be NULL.  Synchronises the stream before returning.  Where the read-out runs
- * on the TMA kernel its waits are bounded: LBM_ETIMEOUT if one gave up, in this call or in earlier steps
- * that did not report it (check_nonfinite 0).  The fields are then not valid; after a wait of the read-out
- * itself the state is as before and the call can be made again.
+ * on the TMA kernel its waits are bounded: LBM_ETIMEOUT if one gave up.  The fields are then not valid;
+ * the state is as before and the call can be made again.
  * Errors: LBM_ESTATE, LBM_ECUDA, LBM_ETIMEOUT. */
 int lbm_get_moments(lbm_ctx* ctx, float* rho, float* ux, float* uy, float* uz, float* T);
 

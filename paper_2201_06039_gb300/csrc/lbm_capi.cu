@@ -13,6 +13,7 @@
 #include "../../include/lbm.h"
 #include "lbm_host.h"
 #include "lbm_launch.h"
+#include "lbm_pool.h"
 
 using namespace gb300lbm;
 
@@ -71,6 +72,16 @@ Layout layout_of(const lbm_params* p, const DevParams& dp) {
     return L;
 }
 
+int* alloc_mapped(size_t bytes) {
+    void* p = nullptr;
+    if (cudaHostAlloc(&p, bytes, cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return (int*)p;   // unified addressing: the device uses the same pointer
+}
+StatusWords g_words(alloc_mapped);
+
 const int kGraphCache = 8;
 
 // A captured run of n steps: what it holds, beyond the buffers, maps and parameters of the context, is
@@ -101,6 +112,7 @@ struct lbm_ctx {
     int variant;   // LBM_KERNEL_TWO_PASS or LBM_KERNEL_FUSED
     TmaMaps maps;
     TmaMaps read_maps;             // of the read-out's tile shape
+    int* gave_up;                  // status word of the TMA read-out (null: it is not used)
     int plan_shape, plan_zchunk;   // TMA plan pinned by lbm_select_plan (-1 / 0: automatic)
     GraphEntry graphs[kGraphCache];
     int n_graphs;
@@ -493,7 +505,7 @@ bool gb300lbm::build_read_maps(const DevParams& d, int precision, void* buf0, vo
     maps->ok = false;
     int shape = -1, zchunk = 0, items = 0;
     tma_plan_for(d, step.sms, tma_read_shape(), 0, 1 << 30, &shape, &zchunk, &items);
-    if (!step.ok || shape < 0) return false;
+    if (!step.ok || shape < 0 || !tma_reads(d)) return false;
     maps->shape = shape;
     maps->zchunk = zchunk;
     maps->items = items;
@@ -649,8 +661,9 @@ int lbm_create(const lbm_params* p, lbm_ctx** out) {
     c->plan_shape = -1;
     c->plan_zchunk = 0;
     c->dp.check_flag = (int*)(c->base + c->L.flag);
-    if (c->variant == LBM_KERNEL_FUSED && p->use_tma != 0 && make_tma_maps(c))
-        build_read_maps(c->dp, c->p.precision, c->pbuf(0), c->pbuf(1), c->maps, &c->read_maps);
+    if (c->variant == LBM_KERNEL_FUSED && p->use_tma != 0 && make_tma_maps(c) &&
+        build_read_maps(c->dp, c->p.precision, c->pbuf(0), c->pbuf(1), c->maps, &c->read_maps))
+        c->gave_up = g_words.take();   // (none left: the generic read-out)
     cudaError_t e = cudaMemsetAsync(c->base + c->L.sums, 0, c->L.flag + sizeof(int) - c->L.sums, c->stream);
     if (e == cudaSuccess && c->dp.wet) {   // scheme 0: the table is constant; scheme 1: refreshed every step
         c->dp.wall_tab = (const float2*)(c->base + c->L.wall);
@@ -663,6 +676,7 @@ int lbm_create(const lbm_params* p, lbm_ctx** out) {
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) {
+        g_words.give(c->gave_up);
         if (c->owns) cudaFree(c->base);
         free(c);
         return fail(LBM_ECUDA, "initial memset: %s", cudaGetErrorString(e));
@@ -760,20 +774,16 @@ int lbm_get_moments(lbm_ctx* c, float* rho, float* ux, float* uy, float* uz, flo
     float* outs[5] = {rho, ux, uy, uz, T};
     float* dst[5];
     for (int k = 0; k < 5; ++k) dst[k] = outs[k] ? (is_device_ptr(outs[k]) ? outs[k] : stage + k * N) : nullptr;
-    bool bounded_waits = false;
+    if (c->gave_up) *c->gave_up = 0;
     CK(launch_readout(c->dp, c->p.precision, B, c->sums(c->slot), dst[0], dst[1], dst[2], dst[3], dst[4], c->stream,
-                      c->maps.ok ? &c->read_maps : nullptr, &bounded_waits));
-    if (bounded_waits && c->dp.test_stall == 2) c->dp.test_stall = 0;   // one stalled read-out only
-    int flag = 0;
-    if (bounded_waits)
-        CK(cudaMemcpyAsync(&flag, c->base + c->L.flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+                      c->maps.ok ? &c->read_maps : nullptr, c->gave_up));
     for (int k = 0; k < 5; ++k)
         if (outs[k] && dst[k] != outs[k])
             CK(cudaMemcpyAsync(outs[k], dst[k], N * 4, cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
-    if (flag & 2) {   // reported here; the flag word's other bits (its low byte) stay for lbm_step
-        CK(cudaMemsetAsync(c->base + c->L.flag, flag & ~2, 1, c->stream));
-        return fail(LBM_ETIMEOUT, "a bounded pipeline wait gave up: the fields are not valid (step %lld)", c->steps);
+    if (c->gave_up && *(volatile int*)c->gave_up) {
+        if (c->dp.test_stall == 2) c->dp.test_stall = 0;   // one stalled read-out only
+        return fail(LBM_ETIMEOUT, "a bounded pipeline wait of the read-out gave up (step %lld)", c->steps);
     }
     return LBM_OK;
 }
@@ -1028,6 +1038,7 @@ void lbm_destroy(lbm_ctx* c) {
     drop_graphs(c);
     if (c->capture) cudaStreamDestroy(c->capture);
     if (c->owns && c->base) cudaFree(c->base);
+    g_words.give(c->gave_up);
     free(c);
 }
 

@@ -414,6 +414,7 @@ __device__ __forceinline__ void back_transform(float rho, float ax, float bx, fl
 // ---------------------------------------------------------------- read-out
 struct ReadFields {   // device arrays, each nullable
     float *rho, *ux, *uy, *uz, *T;
+    int* gave_up;     // TMA read-out: set to 1 if a bounded wait gave up (mapped host memory)
 };
 // the fields of one node (dense index d): u = (j + F/2) / rho, F = F_m + (rho - rho_ave) g from the stencil
 // sums (sx, sy, sz)

@@ -834,12 +834,17 @@ k_fused_tma(const __grid_constant__ CUtensorMap map14, const __grid_constant__ C
     const int ntiles = tiles_x * tiles_y;
     // bounded wait for the bytes of a stage use: a timeout raises the abort flag, after which no
     // role waits for a copy again
-    auto wait_full = [&](int s, unsigned parity) {
-        if (abort_flag) return;
-        if (!mbar_wait(&full_bar[s], parity)) {
-            abort_flag = 1;
+    auto give_up = [&] {
+        abort_flag = 1;
+        if constexpr (kRead) {   // a word the host reads after its synchronisation, without a copy
+            *(volatile int*)out.gave_up = 1;
+            __threadfence_system();
+        } else {
             atomicOr(flag, 2);
         }
+    };
+    auto wait_full = [&](int s, unsigned parity) {
+        if (!abort_flag && !mbar_wait(&full_bar[s], parity)) give_up();
     };
     auto stage_of = [&](int s) { return reinterpret_cast<const S*>(smem_raw + (size_t)s * Sh::kStageOne); };
 
@@ -871,10 +876,7 @@ k_fused_tma(const __grid_constant__ CUtensorMap map14, const __grid_constant__ C
                 if (P.test_stall == (kRead ? 2 : 1) && kl == 0) {
                     // timeout-path test: the first stage's data never comes; the copy warp waits
                     // (bounded) on a barrier nothing completes, then releases the stage empty
-                    if (!mbar_wait(&stall_bar, 0u)) {
-                        abort_flag = 1;
-                        atomicOr(flag, 2);
-                    }
+                    if (!mbar_wait(&stall_bar, 0u)) give_up();
                     mbar_arrive(&full_bar[s]);
                 } else if (abort_flag) {
                     mbar_arrive(&full_bar[s]);   // release the waiters without data
@@ -1495,33 +1497,35 @@ static int zchunk_readout(const DevParams& P, long long tiles) {
     return zc;
 }
 
+// The TMA kernel's read-out instantiation (maps of kReadShape) where its copies pay: from 2^17 nodes
+// (32^3 24 us a call against k_readout's 22, 64 x 64 x 96 33 against 39, 200 x 200 x 300 369 against 527), and
+// not for a frozen g, whose planes z - 1 and z + 1 it would fetch for nothing (181 against 174).  Walls or
+// outflow across x or y, whose patches weigh more there, need planes to make up for them (closed boxes
+// of 512 x 512 x 4 89 against 83, in BF16 87 against 79; of 200 x 200 x 8 42 against 43, 46 against 44; of
+// 96^3 59 against 69, 62 against 65).
+bool tma_reads(const DevParams& P) {
+    const bool faces = (P.xy_walls | P.xy_open) != 0;
+    return P.N >= 1 << 17 && !(faces && P.nz <= 8) && !P.thermal_off;
+}
+
 cudaError_t launch_readout(const DevParams& P, int precision, const StateBufs& B, const double* sums_cur, float* rho,
                            float* ux, float* uy, float* uz, float* T, cudaStream_t s, const TmaMaps* maps,
-                           bool* bounded_waits) {
-    *bounded_waits = false;
+                           int* gave_up) {
     // Thin lattices of some size: a psi pass and a moments pass.  A block that marches planes reads two more
     // than it writes, which a few planes do not repay: 512 x 512 x 1 k_readout 44 us a call, two passes 37;
     // 512 x 512 x 2 54, 47; D3Q19 temperature 87, 77; below 2^16 nodes the second launch costs as much (64 x 64 x 1
     // 25, 27).
     if (P.nz <= 3 && P.N >= 1 << 16) {
         const cudaError_t e = launch_psi(P, precision, B, nullptr, s);
-        return e != cudaSuccess ? e : launch_moments(P, precision, B, sums_cur, ReadFields{rho, ux, uy, uz, T}, s);
+        return e != cudaSuccess ? e : launch_moments(P, precision, B, sums_cur, ReadFields{rho, ux, uy, uz, T, nullptr}, s);
     }
-    // The TMA kernel's read-out instantiation (maps of kReadShape) where its copies pay: from 2^17 nodes
-    // (32^3 24 us a call against k_readout's 22, 64 x 64 x 96 33 against 39, 200 x 200 x 300 369 against 527), and
-    // not for a frozen g, whose planes z - 1 and z + 1 it would fetch for nothing (181 against 174).  Walls or
-    // outflow across x or y, whose patches weigh more there, need planes to make up for them (closed boxes
-    // of 512 x 512 x 4 89 against 83, in BF16 87 against 79; of 200 x 200 x 8 42 against 43, 46 against 44; of
-    // 96^3 59 against 69, 62 against 65).
-    const bool faces = (P.xy_walls | P.xy_open) != 0;
-    if (maps && maps->ok && P.N >= 1 << 17 && !(faces && P.nz <= 8) && !P.thermal_off && tma_runs(P, precision, B)) {
+    if (maps && maps->ok && gave_up && tma_runs(P, precision, B)) {   // (see tma_reads)
         constexpr int TXR = kTmaTX[kReadShape], TYR = kTmaTY[kReadShape];
         const int txs = (P.nx + TXR - 1) / TXR, tys = (P.ny + TYR - 1) / TYR;
         const int ctas = maps->sms < maps->items ? maps->sms : maps->items, first = 0;
         double* sums_next = nullptr;
-        const ReadFields fields{rho, ux, uy, uz, T};
+        const ReadFields fields{rho, ux, uy, uz, T, gave_up};
         cudaError_t e = cudaSuccess;
-        *bounded_waits = true;
         if (precision == 0 && P.wet) GB300_TMA(TXR, TYR, float, true, false, true)
         else if (precision == 0) GB300_TMA(TXR, TYR, float, false, false, true)
         else if (precision == 1) GB300_TMA(TXR, TYR, __nv_bfloat16, false, false, true)
@@ -1533,7 +1537,7 @@ cudaError_t launch_readout(const DevParams& P, int precision, const StateBufs& B
     const dim3 grid(tiles_x, tiles_y, (P.nz + zc - 1) / zc);
 #define GB300_READ(S, QT)                                                                                      \
     k_readout<S, QT, false><<<grid, FusedShape<kTY, QT>::kThreads, 0, s>>>(                                    \
-        P, nullptr, nullptr, (const S*)B.src, B.pull_f, B.pull_g, sums_cur, zc, ReadFields{rho, ux, uy, uz, T}, B.flag)
+        P, nullptr, nullptr, (const S*)B.src, B.pull_f, B.pull_g, sums_cur, zc, ReadFields{rho, ux, uy, uz, T, nullptr}, B.flag)
     if (P.qt == 19) {
         if (precision != 0) return cudaErrorInvalidValue;
         GB300_READ(float, 19);
@@ -1554,7 +1558,7 @@ cudaError_t launch_readout_batch(const DevParams& P, int precision, const BatchI
                                  float* uy, float* uz, float* T, cudaStream_t s) {
 #define GB300_READ(S)                                                                                          \
     k_readout<S, 7, true><<<n_items, FusedShape<kTY>::kThreads, 0, s>>>(                                       \
-        P, insts, items, (const S*)B.src, B.pull_f, B.pull_g, sums_cur, 0, ReadFields{rho, ux, uy, uz, T}, B.flag)
+        P, insts, items, (const S*)B.src, B.pull_f, B.pull_g, sums_cur, 0, ReadFields{rho, ux, uy, uz, T, nullptr}, B.flag)
     switch (precision) {
     case 0: GB300_READ(float); break;
     case 1: GB300_READ(__nv_bfloat16); break;

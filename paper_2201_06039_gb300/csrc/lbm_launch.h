@@ -76,7 +76,7 @@ bool build_tma_maps(const DevParams& d, int precision, void* buf0, void* buf1, i
                     int forced_zchunk, int max_items, TmaMaps* maps);
 
 // Load maps and plan of the read-out (tile shape tma_read_shape(), no partial sums) beside the step's
-// maps of the same lattice and buffers.
+// maps of the same lattice and buffers; false if the lattice is not read out by the TMA kernel.
 bool build_read_maps(const DevParams& d, int precision, void* buf0, void* buf1, const TmaMaps& step, TmaMaps* maps);
 
 // fused z-marching variant (psi of the tile halo recomputed from the populations); uses the
@@ -113,13 +113,15 @@ int tma_ghost_cols(int precision);
 int tma_tile_h(int shape);
 
 // macroscopic fields of the current state (B.src) into the device arrays given (each nullable); a
-// scheme-1 wetting wall's table must be that of this state.  With maps (of tile shape tma_read_shape())
-// and a state the TMA kernel reads, its read-out instantiation runs, else k_readout; on thin lattices a psi
-// pass (into B.psirho) and a moments pass.  *bounded_waits: the launch has waits that can give up (bit 2 of
-// B.flag), after which the fields are not valid.
+// scheme-1 wetting wall's table must be that of this state.  With maps (of build_read_maps), a status word
+// gave_up (mapped host memory, 0) and a state the TMA kernel reads, its read-out instantiation runs, which sets
+// *gave_up to 1 if a bounded wait gave up: the fields are then not valid.  Else k_readout, or on thin
+// lattices a psi pass (into B.psirho) and a moments pass.
 cudaError_t launch_readout(const DevParams& P, int precision, const StateBufs& B, const double* sums_cur, float* rho,
                            float* ux, float* uy, float* uz, float* T, cudaStream_t s, const TmaMaps* maps,
-                           bool* bounded_waits);
+                           int* gave_up);
+// does the read-out of such lattices take the TMA kernel (once the state is in the form it reads)
+bool tma_reads(const DevParams& P);
 int tma_read_shape();
 
 // deterministic FP64 sum of a float field into out[0] (out[1] = 0).
