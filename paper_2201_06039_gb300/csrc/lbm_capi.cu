@@ -463,8 +463,9 @@ int check_flag(lbm_ctx* c) {
 
 namespace {
 
-EncodeTiledFn tensor_map_encoder() {   // looked up once a process (a lookup takes tens of microseconds)
-    static const EncodeTiledFn fn = [] {
+EncodeTiledFn tensor_map_encoder() {   // a lookup takes tens of microseconds: one that succeeded is kept
+    static std::atomic<EncodeTiledFn> kept{nullptr};
+    return kept_lookup(kept, [] {
         void* f = nullptr;
         cudaDriverEntryPointQueryResult q;
         if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
@@ -473,8 +474,7 @@ EncodeTiledFn tensor_map_encoder() {   // looked up once a process (a lookup tak
             f = nullptr;
         }
         return (EncodeTiledFn)f;
-    }();
-    return fn;
+    });
 }
 
 CUtensorMapDataType map_type(int precision) {

@@ -2,6 +2,7 @@
 #pragma once
 #include <stddef.h>
 
+#include <atomic>
 #include <mutex>
 
 namespace gb300lbm {
@@ -44,5 +45,13 @@ private:
     bool used_[kWords] = {};
     int next_ = 0;
 };
+
+// The result of a lookup (a pointer), kept once it is found: a lookup that fails (nullptr) is made again by
+// the next caller.
+template <class Fn, class Lookup> Fn kept_lookup(std::atomic<Fn>& kept, Lookup lookup) {
+    Fn fn = kept.load(std::memory_order_acquire);
+    if (!fn && (fn = lookup())) kept.store(fn, std::memory_order_release);
+    return fn;
+}
 
 }  // namespace gb300lbm
