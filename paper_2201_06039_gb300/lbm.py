@@ -468,14 +468,19 @@ class Lattice:
     def select_plan(self, shape: int, zchunk: int = 0):
         lbm_select_plan(self.ctx, shape, zchunk)
 
+    # revision of the TMA kernel's costs: a plan that was timed on another one is timed again (1: plans
+    # of at least 16 planes a chunk, which leave small lattices at four times their present step)
+    PLAN_REVISION = 2
+
     def plan_key(self) -> str:
-        """Cache key of the plan choice: lattice size, storage, faces, wetting wall and the GPU."""
+        """Cache key of the plan choice: what selects the instantiation of the TMA kernel and its costs
+        (lattice size, storage, faces, wetting wall, frozen temperature), the plan revision and the GPU."""
         import torch
         p = self.params
         wet = int(p.wall_scheme == 1 or p.wall_rho > 0)
         dev = torch.cuda.get_device_name(torch.cuda.current_device()).replace(" ", "_")
         return (f"{p.nx}x{p.ny}x{p.nz}/prec{p.precision}/bc{''.join(str(int(b)) for b in p.bc)}"
-                f"/wet{wet}/{dev}")
+                f"/wet{wet}/frozen{int(bool(p.thermal_off))}/plan{self.PLAN_REVISION}/{dev}")
 
     def autotune(self, steps: int = 10, cache: str = None) -> dict:
         """Pick the TMA plan by timing (lbm_autotune), or take it from the JSON file `cache` if that
