@@ -1247,6 +1247,22 @@ __global__ void __launch_bounds__(256) k_ghosts(DevParams P, S* __restrict__ pop
     }
 }
 
+}  // namespace
+
+// SM count of the current device (queried once per device)
+int device_sms() {
+    static int cached[64] = {0};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return 1;
+    if (dev < 64 && cached[dev] > 0) return cached[dev];
+    int n = 0;
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 1;
+    if (dev < 64) cached[dev] = n;
+    return n;
+}
+
+namespace {
+
 // Tile shapes of the TMA kernel (index = plan shape): 8 to 13 compute warps of one tile node a
 // thread.  kTmaRate is each shape's node rate per CTA relative to 32 x 8, measured (a plane of a tile
 // takes 1.75, 2.3, 2.26, 2.51, 2.4, 2.53 us on the pool, 1.97 us for one 32 x 8 tile alone).  The 40-wide
@@ -1302,18 +1318,6 @@ void tma_plan(const DevParams& P, int ctas, int forced_shape, int forced_zchunk,
             }
         }
     }
-}
-
-// SM count of the current device (queried once per device)
-int device_sms() {
-    static int cached[64] = {0};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return 1;
-    if (dev < 64 && cached[dev] > 0) return cached[dev];
-    int n = 0;
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 1;
-    if (dev < 64) cached[dev] = n;
-    return n;
 }
 
 int zchunk_generic(const DevParams& P, int tiles) {
@@ -1570,6 +1574,7 @@ cudaError_t launch_readout_batch(const DevParams& P, int precision, const BatchI
 #undef GB300_READ
     return cudaGetLastError();
 }
+#undef GB300_TMA
 
 int batch_tile_rows(int ty) { return ty == 4 ? 4 : kTY; }
 

@@ -313,7 +313,8 @@ cudaError_t launch_init(const DevParams& P, int precision, void* pops, const flo
 cudaError_t launch_psi(const DevParams& P, int precision, const StateBufs& B, double* sums, cudaStream_t s) {
     dim3 blk(TPB_X, TPB_Y), grid = grid_of(P);
     // with sums: one round of three blocks an SM, at most 16 planes a block; without, a plane a block
-    const int zc = !sums ? 1 : (int)std::max(1LL, std::min(16LL, ((long long)grid.x * grid.y * grid.z + 455) / 456));
+    const long long round = 3LL * device_sms(), planes = ((long long)grid.x * grid.y * grid.z + round - 1) / round;
+    const int zc = !sums ? 1 : (int)std::max(1LL, std::min(16LL, planes));
     grid.z = (P.nz + zc - 1) / zc;
     GB300_DISPATCH_QT(P, precision, (k_psi<S, QT><<<grid, blk, 0, s>>>(P, (const S*)B.src, B.pull_f, B.pull_g, B.psirho,
                                                                        B.partial, B.counter, sums, B.flag, zc)));

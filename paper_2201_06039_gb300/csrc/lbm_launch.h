@@ -131,6 +131,7 @@ cudaError_t launch_sum_field(const float* a, int n, double2* partial, unsigned* 
                              double* out, cudaStream_t s);
 
 int max_partials(const DevParams& P);
+int device_sms();   // of the current device
 
 // ---------------------------------------------------------------- batched ensemble
 // Geometry of one instance (device table).  Instance k owns the elements [pop_off, pop_off + its
