@@ -194,7 +194,7 @@ double busiest_stream(std::vector<double> t) {
 // generic kernel's rate, 12500 nodes a microsecond in 32 x 8 tiles, and the columns' share of the SMs bound
 // the two for many.  Measured, TMA against generic, us a step: closed boxes 1 x 32^3 89 / 33, 64 x 32^3
 // 211 / 182, 2 x (64 x 64 x 70) 99 / 54, 4 x 101 / 89, 5 x 104 / 111, 8 x 127 / 175, 3 x 96^3 153 / 192, 16 x
-// (20 x 20 x 100) 139 / 94, 32 x 154 / 184; frozen 1 x 32^3 96 / 30, 8 x (64 x 64 x 70) 157 / 156, 3 x 96^3 159 / 174.
+// (20 x 20 x 100) 139 / 94, 32 x 154 / 184, 256 x 8^3 (a tie here) 191 / 221; frozen 1 x 32^3 96 / 30, 8 x (64 x 64 x 70) 157 / 156, 3 x 96^3 159 / 174.
 bool columns_pay(const lbm_batch* b) {
     std::vector<double> col(b->n), gen(b->n);
     double col_work = 0.0, gen_nodes = 0.0;
@@ -206,7 +206,7 @@ bool columns_pay(const lbm_batch* b) {
         col_work += m.ok ? col[k] * m.items : 0.0;
         gen_nodes += (double)((d.nx + 31) / 32 * 32) * ((d.ny + 7) / 8 * 8) * d.nz;
     }
-    return std::max(busiest_stream(col), col_work / b->sms) < std::max(busiest_stream(gen), gen_nodes / 12500.0);
+    return std::max(busiest_stream(col), col_work / b->sms) <= std::max(busiest_stream(gen), gen_nodes / 12500.0);
 }
 
 // TMA mode: tensor maps and plan of every instance: whole- or half-column items and the tile shape with
