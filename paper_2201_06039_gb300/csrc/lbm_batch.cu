@@ -236,8 +236,8 @@ int set_tma_plan(lbm_batch* b) {
         const DevParams& d = b->dps[k];
         const size_t po = (size_t)b->inst[k].pop_off * pb;
         // tall columns in two halves: a step of an instance is one launch, as long as its longest item
-        // (4.81 -> 4.64 ms a step on 256 instances of edges 24..96; the halves' two extra planes do not pay
-        // below 60 planes)
+        // (4.81 -> 4.62 ms a step on 256 cubes of edges 24..96 and 72.9M nodes, in calls of 5 steps as of 200;
+        // the halves' two extra planes do not pay below 60 planes)
         const bool tma = build_tma_maps(d, b->p.precision, b->pbuf(0) + po, b->pbuf(1) + po, 1, -1,
                                         d.nz > 60 ? (d.nz + 1) / 2 : d.nz, b->t_cap[k], &b->tmaps[k]);
         if (!tma && !fused_supported(d))
@@ -693,7 +693,7 @@ int lbm_batch_autotune(lbm_batch* b, int steps, double* best_ms) {
         if (rc) break;
         rc = enqueue_batch_step(b);   // warm-up
         // the TMA mode as lbm_batch_step runs it, one replayed chain: a few directly enqueued steps with a
-        // fork and join measured 5.17 ms a step where replayed chains run at 4.33
+        // fork and join measured 5.17 ms a step where replayed chains run at 4.33 (256 instances, 66.3M nodes)
         const bool chain = q == kTmaPlan && b->p.use_graph;
         const int m = q == kTmaPlan ? kTmaChain : steps;
         if (chain && rc == LBM_OK) rc = run_batch_graph(b, m);
