@@ -50,26 +50,18 @@ struct Layout {
     size_t pops[2], psirho, phis, sums, partial, counter, flag, vel, wall, wpar, wbad, total;
 };
 
-// the variant a context of p runs (kernel AUTO resolved)
-int variant_of(const lbm_params* p, const DevParams& dp) {
-    if (p->kernel != LBM_KERNEL_AUTO) return p->kernel;
-    return fused_supported(dp) && p->divu_mode == 0 ? LBM_KERNEL_FUSED : LBM_KERNEL_TWO_PASS;
-}
-
-// does a context of p hold the (psi, rho) field: the two-pass step and the read-out of thin lattices do
-bool keeps_psirho(const lbm_params* p, const DevParams& dp) {
-    return variant_of(p, dp) == LBM_KERNEL_TWO_PASS || thin_readout(dp);
-}
-
 // Device memory of a context: two population buffers (rows of 26 or 38 slots: the padded,
-// ghost-carrying storage of lbm_device.cuh), dense (psi, rho) where used and phi_s fields, FP64 sums.
+// ghost-carrying storage of lbm_device.cuh), dense (psi, rho) and phi_s fields, FP64 sums.
+// (psi, rho) is written by the two-pass variant and the read-out of thin lattices only, but its room stays
+// in every context: with phi_s moved up into it the unchanged TMA kernel ran slower on small lattices
+// (32^3 12.12 -> 12.41 us a step, 41 x 29 x 25 15.14 -> 15.53).
 Layout layout_of(const lbm_params* p, const DevParams& dp) {
     Layout L;
     size_t N = (size_t)dp.N, pb = pop_bytes(p->precision), off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off = align256(off + bytes); return o; };
     L.pops[0] = take(pop_elems(dp) * pb);
     L.pops[1] = take(pop_elems(dp) * pb);
-    L.psirho = take(keeps_psirho(p, dp) ? 8 * N : 0);
+    L.psirho = take(8 * N);
     L.phis = take(4 * N);
     L.sums = take(8 * sizeof(double));          // slots: [0..1] [2..3] rho_ave ping-pong, [4..5] totals
     L.partial = take(sizeof(double2) * (size_t)max_partials(dp));
@@ -138,7 +130,7 @@ struct lbm_ctx {
         B.src_index = cur;
         B.pull_f = fresh_f ? 0 : 1;
         B.pull_g = fresh_g ? 0 : 1;
-        B.psirho = keeps_psirho(&p, dp) ? (float2*)(base + L.psirho) : nullptr;
+        B.psirho = (float2*)(base + L.psirho);
         B.phis = (float*)(base + L.phis);
         B.partial = (double2*)(base + L.partial);
         B.counter = (unsigned*)(base + L.counter);
@@ -661,7 +653,9 @@ int lbm_create(const lbm_params* p, lbm_ctx** out) {
         }
         c->owns = true;
     }
-    c->variant = variant_of(p, c->dp);
+    c->variant = p->kernel == LBM_KERNEL_AUTO
+                     ? (fused_supported(c->dp) && p->divu_mode == 0 ? LBM_KERNEL_FUSED : LBM_KERNEL_TWO_PASS)
+                     : p->kernel;
     if (c->variant == LBM_KERNEL_FUSED && !fused_supported(c->dp)) {
         if (c->owns) cudaFree(c->base);
         free(c);

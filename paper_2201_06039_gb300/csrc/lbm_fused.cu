@@ -1514,16 +1514,14 @@ bool tma_reads(const DevParams& P) {
     return P.N >= 1 << 17 && !(faces && P.nz <= 8) && !P.thermal_off;
 }
 
-// Thin lattices of some size: a psi pass and a moments pass.  A block that marches planes reads two more
-// than it writes, which a few planes do not repay: 512 x 512 x 1 k_readout 44 us a call, two passes 37;
-// 512 x 512 x 2 54, 47; D3Q19 temperature 87, 77; below 2^16 nodes the second launch costs as much (64 x 64 x 1
-// 25, 27).
-bool thin_readout(const DevParams& P) { return P.nz <= 3 && P.N >= 1 << 16; }
-
 cudaError_t launch_readout(const DevParams& P, int precision, const StateBufs& B, const double* sums_cur, float* rho,
                            float* ux, float* uy, float* uz, float* T, cudaStream_t s, const TmaMaps* maps,
                            int* gave_up) {
-    if (thin_readout(P)) {
+    // Thin lattices of some size: a psi pass and a moments pass.  A block that marches planes reads two more
+    // than it writes, which a few planes do not repay: 512 x 512 x 1 k_readout 44 us a call, two passes 37;
+    // 512 x 512 x 2 54, 47; D3Q19 temperature 87, 77; below 2^16 nodes the second launch costs as much (64 x 64 x 1
+    // 25, 27).
+    if (P.nz <= 3 && P.N >= 1 << 16) {
         const cudaError_t e = launch_psi(P, precision, B, nullptr, s);
         return e != cudaSuccess ? e : launch_moments(P, precision, B, sums_cur, ReadFields{rho, ux, uy, uz, T, nullptr}, s);
     }

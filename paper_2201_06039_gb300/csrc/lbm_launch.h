@@ -13,7 +13,7 @@ struct StateBufs {
     void* dst;             // populations written this step
     int src_index;         // which of the two population buffers src is (tensor maps are per buffer)
     int pull_f, pull_g;    // 0: state is post-streaming at the node (right after init)
-    float2* psirho;        // per node (psi, rho): two-pass step and thin read-out only, else NULL
+    float2* psirho;        // per node (psi, rho)
     float* phis;           // phi_s history, read and rewritten in place
     double2* partial;      // per-block partial sums of the deterministic reduction
     unsigned* counter;     // last-block counter of the reduction (kept at 0 between launches)
@@ -122,8 +122,6 @@ cudaError_t launch_readout(const DevParams& P, int precision, const StateBufs& B
                            int* gave_up);
 // does the read-out of such lattices take the TMA kernel (once the state is in the form it reads)
 bool tma_reads(const DevParams& P);
-// is the read-out of such lattices a psi pass and a moments pass (B.psirho needed)
-bool thin_readout(const DevParams& P);
 int tma_read_shape();
 
 // deterministic FP64 sum of a float field into out[0] (out[1] = 0).
